@@ -57,7 +57,9 @@ extern "C" {
 #define GB_ETIMEOUT -3   /* a persistent kernel stopped at the context's time budget */
 #define GB_ENOMEM   -4   /* device allocation failed */
 
-#define GB_FP64   0      /* every step in IEEE double */
+#define GB_FP64   0      /* double precision: set-up, inner products and outputs in IEEE
+                            double; response samples and FFT in 64-bit fixed point (58 or
+                            more fractional bits) where the parameters allow, else double */
 #define GB_MIXED  1      /* carrier phase modulo one cycle in 64-bit fixed point
                             (double-word float arithmetic for candidates outside
                             its ranges), per-candidate set-up and carrier offset

@@ -81,6 +81,16 @@ struct TabSet64 {
 struct TabSet32 {
     OrbitTables32 t[kNumSizes];
 };
+// Fixed-point tables of the FP64 path (fx64.cuh): per size [4][N] int4 of two
+// Q62 values each, (n01.x, n01.y), (n01.z, n12.x), (n12.y, n12.z), (cos a, sin
+// a), and the twiddles cos, sin 2 pi k/1024, k < kTwiddles.
+struct FxTw;
+struct TabSetFx {
+    const int4* geo[kNumSizes];
+    const FxTw* tw;
+    double arm_c;        // L/c, s
+    int krho_q30;        // (L/c)/(3 1024 s) in Q30
+};
 
 // Work item: candidates [c_begin, c_end) of window `win`.
 struct Tile {
@@ -138,6 +148,7 @@ struct gb_ctx {
     double* d_tab64[gb::kNumSizes] = {};
     float* d_tab32[gb::kNumSizes] = {};
     double* d_tw64 = nullptr;   // kTwiddles complex
+    int4* d_fx = nullptr;       // fixed-point tables of every N, then the twiddles
     float* d_tw32 = nullptr;
     int* d_status = nullptr;    // device status word (GB_OK or GB_EINVAL)
     std::vector<gb::Plan> plans;
@@ -217,6 +228,7 @@ OrbitTables64 tables64(const gb_ctx* ctx, int N);
 OrbitTables32 tables32(const gb_ctx* ctx, int N);
 TabSet64 tabset64(const gb_ctx* ctx);
 TabSet32 tabset32(const gb_ctx* ctx);
+TabSetFx tabset_fx(const gb_ctx* ctx);
 inline double transfer_frequency(const gb_ctx* ctx) { return kC / (2.0 * kPi * ctx->obs.arm_L); }
 
 // Validate windows and return (creating and uploading if needed) the launch

@@ -1,0 +1,93 @@
+"""The FP64 path's fixed-point slow part and transform at the edges of its ranges.
+
+Candidates on both sides of each range (series tiers at f_max/f* = 1/2 and
+1.3, drift f0/1024, f0 <= 0) and every template length, against the model in
+long double.  The tolerance is the rounding of phases in double: a handful of
+roundings (8) of terms of the size of f0 k.x/c, fdot T^2/2 and phi0/2pi
+cycles, times 2 pi, on top of 1e-14 for the response."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import gb
+from paper_2307_03763_gb300 import api
+from paper_2307_03763_gb300 import workloads as wk
+
+from tests import _longdouble as ld
+
+pytestmark = pytest.mark.gpu
+
+FSTAR = gb.transfer_frequency()
+
+
+def candidates(f0, fdot, n, seed):
+    rng = np.random.default_rng(seed)
+    th = np.empty((n, 8))
+    th[:, 0] = f0
+    th[:, 1] = fdot
+    th[:, 2], th[:, 3], th[:, 5], th[:, 6], th[:, 7] = wk.random_angles(rng, n)
+    th[:, 4] = np.exp(rng.uniform(math.log(1e-23), math.log(1e-21), n))
+    th[0, 2], th[1 % n, 2] = math.pi / 2, -math.pi / 2
+    return th
+
+
+def tolerance(th, T):
+    cycles = np.abs(th[:, 0]) * 510.0 + np.abs(0.5 * th[:, 1]) * T * T + np.abs(th[:, 7]) / (2 * math.pi) + 1.0
+    return 8 * 2 * math.pi * 2.0 ** -53 * cycles + 1e-14
+
+
+CASES = [(0.3e-3, 0.0, 32), (1e-3, 1e-18, 64), (0.4995 * FSTAR, 1e-15, 128), (0.5005 * FSTAR, 1e-15, 256),
+         (1.299 * FSTAR, 2e-13, 512), (1.301 * FSTAR, 2e-13, 256), (2.0 * FSTAR, 0.0, 64), (3.0 * FSTAR, 0.0, 64),
+         (15e-3, 1.2e-13, 1024), (20e-3, 9e-13, 1024), (5e-3, -3e-14, 128),
+         (1e-3, 0.999e-3 / (1024 * wk.YEAR), 64), (1e-3, 1.001e-3 / (1024 * wk.YEAR), 64),
+         (-2e-3, 1e-17, 64), (0.0, 0.0, 32)]
+
+
+@pytest.mark.parametrize("f0,fdot,N", CASES)
+def test_templates_at_range_edges(f0, fdot, N):
+    T = wk.YEAR
+    th = candidates(f0, fdot, 7, int(N))
+    ctx = api.Context(T)
+    out = ctx.waveform_aet(torch.as_tensor(th, device="cuda"), N)
+    q, ref = ld.template_aet(th, N, T)
+    assert np.array_equal(out[3].cpu().numpy(), q)
+    tol = tolerance(th, T)
+    norm = lambda x: np.sqrt((np.abs(x) ** 2).sum(1).astype(np.float64))  # noqa: E731
+    for h, r in zip(out[:2], ref[:2]):
+        assert np.all(norm(h.cpu().numpy() - r) <= tol * np.maximum(norm(r), 1e-300))
+    # T is a small difference of terms of A's size in the plain form
+    assert np.all(norm(out[2].cpu().numpy() - ref[2]) <= tol * np.maximum(norm(ref[0]) + norm(ref[1]), 1e-300))
+    ctx.check()
+
+
+@pytest.mark.parametrize("n", [1, 5, 16, 17, 127, 130])
+def test_mixed_forms_in_one_call(n):
+    """Fixed-point and plain-double candidates side by side, counts around a warp's set-up group."""
+    T = 0.5 * wk.YEAR
+    th = candidates(4e-3, 1e-15, n, n)
+    th[::3, 0] = 1.4 * FSTAR       # plain double
+    th[::3, 1] = 0.0
+    N = 128
+    wins = [(int(4e-3 * T) - 64, 128, N, 0, 0, n)]
+    rng = np.random.default_rng(n)
+    d = rng.standard_normal((2, 128, 2)) @ np.array([1, 1j])
+    w = rng.uniform(0.5, 1.5, (2, 128)) * 1e41
+    ctx = api.Context(T)
+    dev = lambda x: torch.as_tensor(x, device="cuda")  # noqa: E731
+    d = d * 1e-20
+    args = [dev(np.ascontiguousarray(x)) for x in (d[0], d[1], w[0], w[1])]
+    got = ctx.loglik(wins, *args, dev(th))
+    ref = [np.asarray(x, dtype=np.float64) for x in ld.loglik(wins[0], d[0], d[1], w[0], w[1], th, T)]
+    tol = tolerance(th, T)
+    dd = -2.0 * float(ref[0][0]) if n > 0 else 0.0   # the first candidate lies outside the window: logL = -<d|d>/2
+    for g, r in zip(got, ref):
+        scale = np.abs(ref[2]) + np.sqrt(np.abs(ref[2]) * dd) + dd
+        assert np.all(np.abs(g.cpu().numpy() - r) <= 2 * tol * scale)
+    # the row list evaluates the same bits
+    rows = torch.arange(n, dtype=torch.int32, device="cuda")
+    lo, hi = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.full((1,), n, dtype=torch.int32, device="cuda")
+    again = ctx.loglik_rows(wins, *args, dev(th), rows, lo, hi)
+    for a, b in zip(again, got):
+        assert torch.equal(a, b)
