@@ -8,9 +8,12 @@ fallback: if ``libgb.so`` is missing the import of the library raises.
 Tensors: theta float64 (n, 8) in the order (f0, fdot, beta, lambda, A, iota,
 psi, phi0); data complex128; weights 1/S float64; all on one CUDA device.
 """
+import array
 import ctypes
+import itertools
 import os
 
+import numpy as np
 import torch
 
 from . import build as _build
@@ -33,6 +36,9 @@ class Window(ctypes.Structure):
     _fields_ = [("k0", ctypes.c_int64), ("data_off", ctypes.c_int64), ("cand_off", ctypes.c_int64),
                 ("W", ctypes.c_int32), ("N", ctypes.c_int32), ("n_cand", ctypes.c_int32),
                 ("reserved", ctypes.c_int32)]
+
+
+_WINDOW_DTYPE = np.dtype([(n, np.int64 if t is ctypes.c_int64 else np.int32) for n, t in Window._fields_])
 
 
 class Obs(ctypes.Structure):
@@ -148,6 +154,32 @@ def windows_array(windows):
     return arr
 
 
+class _Layout:
+    """A window layout as the library takes it: the descriptor array, the rows
+    [0, covered) its candidate ranges cover one after the other (-1 when they
+    leave a gap or overlap) and the most candidates of a window."""
+    __slots__ = ("arr", "n", "covered", "kmax")
+
+    def __init__(self, windows):
+        self.n = len(windows)
+        try:   # integers, converted in bulk
+            if self.n == 0 or set(map(len, windows)) != {6}:
+                raise TypeError
+            t = np.array(array.array("q", itertools.chain.from_iterable(windows)), dtype=np.int64).reshape(self.n, 6)
+            rec = np.zeros(self.n, dtype=_WINDOW_DTYPE)
+            for k, name in enumerate(("k0", "W", "N", "data_off", "cand_off", "n_cand")):
+                rec[name] = t[:, k]
+            self.arr = (Window * self.n).from_buffer_copy(rec)
+        except (TypeError, OverflowError):
+            rows = [tuple(int(x) for x in w) for w in windows]
+            self.arr = windows_array(rows)
+            t = np.array(rows, dtype=np.int64).reshape(self.n, 6)
+        off, cnt = t[:, 4], t[:, 5]
+        gapless = bool((cnt >= 0).all()) and np.array_equal(off, np.cumsum(cnt) - cnt)
+        self.covered = int(cnt.sum()) if gapless else -1
+        self.kmax = int(max(1, cnt.max(initial=1)))
+
+
 class Context:
     """A libgb context on one CUDA device (owns the orbit and twiddle tables)."""
 
@@ -163,7 +195,8 @@ class Context:
         if rc != GB_OK:
             raise GBError(rc, "gb_ctx_create failed")
         self._h = h
-        self._win_cache = {}
+        self._layouts = {}
+        self._budget = False
 
     def close(self):
         if getattr(self, "_h", None):
@@ -183,6 +216,7 @@ class Context:
     def set_time_budget(self, seconds):
         """Work budget of the persistent mixed-precision kernels (0: none)."""
         self._check(lib().gb_ctx_set_time_budget(self._h, float(seconds)))
+        self._budget = float(seconds) > 0.0
 
     def set_kernel_events(self, start, end):
         """Record two torch.cuda.Event objects (timing enabled, recorded at
@@ -203,15 +237,37 @@ class Context:
         """Synchronise and raise if a kernel met a non-finite parameter."""
         self._check(lib().gb_ctx_check(self._h))
 
+    def _layout(self, windows):
+        """The layout of a window list, kept by value: a list whose rows equal a
+        kept one's (tuples of ints; 70 us for 2,048 windows) is not converted
+        again (0.8 ms)."""
+        try:
+            key = tuple(windows)
+            lay = self._layouts.get(key)
+        except TypeError:   # rows that cannot be hashed (lists, arrays)
+            key = lay = None
+        if lay is None:
+            if key is None or not (set(map(type, key)) <= {tuple} and
+                                   set(map(type, itertools.chain.from_iterable(key))) <= {int}):
+                key = tuple(tuple(int(x) for x in w) for w in windows)   # only immutable keys are kept
+                lay = self._layouts.get(key)
+            if lay is None:
+                if len(self._layouts) > 64:
+                    self._layouts.clear()
+                lay = self._layouts[key] = _Layout(key)
+        return lay
+
     def _windows(self, windows):
-        key = tuple(tuple(int(x) for x in w) for w in windows)
-        arr = self._win_cache.get(key)
-        if arr is None:
-            if len(self._win_cache) > 64:
-                self._win_cache.clear()
-            arr = windows_array(windows)
-            self._win_cache[key] = arr
-        return arr, len(windows)
+        lay = self._layout(windows)
+        return lay.arr, lay.n
+
+    def _outputs(self, lay, *shapes):
+        """New float64 outputs.  Rows no window covers read zero, and so do rows a
+        time budget leaves out; where the windows cover every row the kernels
+        write them all and the fill (a launch each) is left out."""
+        full = lay.covered == shapes[0][0] and not self._budget
+        make = torch.empty if full else torch.zeros
+        return tuple(make(s, dtype=torch.float64, device=self.device) for s in shapes)
 
     def waveform(self, theta, N, prec="fp64"):
         """A/E templates on bins q - N/2 .. q + N/2 - 1: returns hA, hE (B, N) complex128, q (B,) int64."""
@@ -232,14 +288,14 @@ class Context:
         _need(wE, torch.float64, self.device, "wE", (nb,))
         n = theta.shape[0] if theta.dim() == 2 else -1
         _need(theta, torch.float64, self.device, "theta", (n, 8))
-        arr, nw = self._windows(windows)
-        return arr, nw, nb, n
+        return self._layout(windows), nb, n
 
     def loglik(self, windows, dA, dE, wA, wE, theta, prec="fp64", out=None):
         """logL, <d|h>, <h|h> per candidate (Eq. 2 over each window)."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         if out is None:
-            out = tuple(torch.zeros(n, dtype=torch.float64, device=self.device) for _ in range(3))
+            out = self._outputs(lay, *([(n,)] * 3))
         logL, dh, hh = out
         for t, name in ((logL, "logL"), (dh, "dh"), (hh, "hh")):
             if t is not None:
@@ -250,11 +306,12 @@ class Context:
 
     def loglik_aet(self, windows, dA, dE, dT, wA, wE, wT, theta, prec="fp64", out=None):
         """logL, <d|h>, <h|h> with the T channel in the windows above f*/2 (see gb_loglik_aet)."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         _need(dT, torch.complex128, self.device, "dT", (nb,))
         _need(wT, torch.float64, self.device, "wT", (nb,))
         if out is None:
-            out = tuple(torch.zeros(n, dtype=torch.float64, device=self.device) for _ in range(3))
+            out = self._outputs(lay, *([(n,)] * 3))
         logL, dh, hh = out
         for t, name in ((logL, "logL"), (dh, "dh"), (hh, "hh")):
             if t is not None:
@@ -266,11 +323,12 @@ class Context:
 
     def loglik_phase_aet(self, windows, dA, dE, dT, wA, wE, wT, theta, prec="fp64", out=None):
         """loglik_phase with the T channel above f*/2 (see gb_loglik_phase_aet)."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         _need(dT, torch.complex128, self.device, "dT", (nb,))
         _need(wT, torch.float64, self.device, "wT", (nb,))
         if out is None:
-            out = tuple(torch.zeros(n, dtype=torch.float64, device=self.device) for _ in range(4))
+            out = self._outputs(lay, *([(n,)] * 4))
         logL, dh, dh_im, hh = out
         _need(dh_im, torch.float64, self.device, "dh_im", (n,))
         for t, name in ((logL, "logL"), (dh, "dh"), (hh, "hh")):
@@ -283,12 +341,12 @@ class Context:
 
     def loglik_grad_aet(self, windows, dA, dE, dT, wA, wE, wT, theta, prec="fp64", out=None):
         """logL and d logL / d theta (n, 8) with the T channel above f*/2 (see gb_loglik_grad_aet)."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         _need(dT, torch.complex128, self.device, "dT", (nb,))
         _need(wT, torch.float64, self.device, "wT", (nb,))
         if out is None:
-            out = (torch.zeros(n, dtype=torch.float64, device=self.device),
-                   torch.zeros((n, 8), dtype=torch.float64, device=self.device))
+            out = self._outputs(lay, (n,), (n, 8))
         logL, grad = out
         if logL is not None:
             _need(logL, torch.float64, self.device, "logL", (n,))
@@ -311,9 +369,10 @@ class Context:
 
     def loglik_phase(self, windows, dA, dE, wA, wE, theta, prec="fp64", out=None):
         """logL, <d|h>, <d|h>_im, <h|h> per candidate (see gb_loglik_phase)."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         if out is None:
-            out = tuple(torch.zeros(n, dtype=torch.float64, device=self.device) for _ in range(4))
+            out = self._outputs(lay, *([(n,)] * 4))
         logL, dh, dh_im, hh = out
         _need(dh_im, torch.float64, self.device, "dh_im", (n,))
         for t, name in ((logL, "logL"), (dh, "dh"), (hh, "hh")):
@@ -326,10 +385,10 @@ class Context:
 
     def loglik_grad(self, windows, dA, dE, wA, wE, theta, prec="fp64", out=None):
         """logL and d logL / d theta (n, 8) by the adjoint kernel."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         if out is None:
-            out = (torch.zeros(n, dtype=torch.float64, device=self.device),
-                   torch.zeros((n, 8), dtype=torch.float64, device=self.device))
+            out = self._outputs(lay, (n,), (n, 8))
         logL, grad = out
         if logL is not None:
             _need(logL, torch.float64, self.device, "logL", (n,))
@@ -341,7 +400,8 @@ class Context:
 
     def autotune(self, windows, dA, dE, wA, wE, theta, prec="mixed", reps=3):
         """Pick the fastest launch shape for this batch (see gb_autotune); returns a dict."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         logL = torch.empty(n, dtype=torch.float64, device=self.device)
         t = Tuning()
         self._check(lib().gb_autotune(self._h, PRECISIONS[prec], arr, nw, _ptr(dA), _ptr(dE), _ptr(wA), _ptr(wE),
@@ -494,7 +554,8 @@ class Context:
     def loglik_rows(self, windows, dA, dE, wA, wE, theta, rows, row_lo, row_hi, out=None):
         """FP64 logL, <d|h>, <h|h> of listed rows (see gb_loglik_rows): window w's entries are
         rows[cand_off + j], j in [row_lo[w], row_hi[w]); the other rows of the outputs are kept."""
-        arr, nw, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, n = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         _need(rows, torch.int32, self.device, "rows", (n,))
         _need(row_lo, torch.int32, self.device, "row_lo", (nw,))
         _need(row_hi, torch.int32, self.device, "row_hi", (nw,))
@@ -515,7 +576,8 @@ class Context:
         (see gb_mh_certified).  Window w holds rows [w n, (w + 1) n).  Returns
         (chain, n_accept, logL, dh, hh, n_exact, pending); pending (1,) int32 is 0 when every
         decision is certified."""
-        arr, nw, nb, nrow = self._data_args(windows, dA, dE, wA, wE, theta)
+        lay, nb, nrow = self._data_args(windows, dA, dE, wA, wE, theta)
+        arr, nw = lay.arr, lay.n
         n = nrow // max(nw, 1)
         for t, name in ((log_g, "log_g"), (log_u, "log_u")):
             _need(t, torch.float64, self.device, name, (nw, n))
@@ -552,9 +614,10 @@ class Context:
             _need(dE, torch.complex128, self.device, "dE", (nb,))
         n = theta.shape[0] if theta.dim() == 2 else -1
         _need(theta, torch.float64, self.device, "theta", (n, 8))
-        arr, nw = self._windows(windows)
+        lay = self._layout(windows)
+        arr, nw = lay.arr, lay.n
         if kmax is None:
-            kmax = max([1] + [int(w[5]) for w in windows])
+            kmax = lay.kmax
         gram = torch.full((nw, kmax, kmax), float("nan"), dtype=torch.float64, device=self.device)
         rho = dh = None
         if dA is not None:

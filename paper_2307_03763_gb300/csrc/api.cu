@@ -17,12 +17,12 @@ int check_windows(gb_ctx* ctx, const char* fn, const gb_window_t* win, int32_t n
     if (n_bins < 0 || n_rows < 0) return set_error(ctx, GB_EINVAL, std::string(fn) + ": negative extent");
     for (int i = 0; i < n_win; ++i) {
         const gb_window_t& w = win[i];
-        const std::string at = std::string(fn) + ": window " + std::to_string(i) + ": ";
-        if (!valid_size(w.N)) return set_error(ctx, GB_EINVAL, at + "N must be a power of two in [32, 1024]");
-        if (w.W < 0 || w.n_cand < 0 || w.data_off < 0 || w.cand_off < 0)
-            return set_error(ctx, GB_EINVAL, at + "negative size or offset");
-        if (w.data_off + (int64_t)w.W > n_bins) return set_error(ctx, GB_EINVAL, at + "data_off + W > n_bins");
-        if (w.cand_off + (int64_t)w.n_cand > n_rows) return set_error(ctx, GB_EINVAL, at + "cand_off + n_cand > n_rows");
+        const char* what = !valid_size(w.N) ? "N must be a power of two in [32, 1024]"
+                           : w.W < 0 || w.n_cand < 0 || w.data_off < 0 || w.cand_off < 0 ? "negative size or offset"
+                           : w.data_off + (int64_t)w.W > n_bins ? "data_off + W > n_bins"
+                           : w.cand_off + (int64_t)w.n_cand > n_rows ? "cand_off + n_cand > n_rows"
+                                                                     : nullptr;
+        if (what) return set_error(ctx, GB_EINVAL, std::string(fn) + ": window " + std::to_string(i) + ": " + what);
         *total += w.n_cand;
     }
     return GB_OK;

@@ -215,12 +215,16 @@ TabSet32 tabset32(const gb_ctx* ctx) {
 // ---------------------------------------------------------------------------
 // launch plans
 // ---------------------------------------------------------------------------
-static uint64_t fnv1a(const void* p, size_t n, uint64_t h) {
+// a hash of n bytes, eight at a time (a lookup compares the layout itself)
+static uint64_t hash_bytes(const void* p, size_t n, uint64_t h) {
     const unsigned char* b = (const unsigned char*)p;
-    for (size_t i = 0; i < n; ++i) {
-        h ^= b[i];
-        h *= 1099511628211ull;
+    for (; n >= 8; n -= 8, b += 8) {
+        uint64_t v;
+        std::memcpy(&v, b, 8);
+        h = (h ^ v) * 0x9E3779B97F4A7C15ull;
+        h ^= h >> 29;
     }
+    for (; n > 0; --n, ++b) h = (h ^ *b) * 1099511628211ull;
     return h;
 }
 
@@ -282,10 +286,10 @@ static void split_last(std::vector<Tile>& v, size_t k) {
 int get_plan(gb_ctx* ctx, int prec, const gb_window_t* win, int32_t n_win, int tile_cands,
              const Plan** out) {
     uint64_t key = 1469598103934665603ull;
-    key = fnv1a(&prec, sizeof prec, key);
-    key = fnv1a(&tile_cands, sizeof tile_cands, key);
-    key = fnv1a(&n_win, sizeof n_win, key);
-    key = fnv1a(win, sizeof(gb_window_t) * (size_t)n_win, key);
+    key = hash_bytes(&prec, sizeof prec, key);
+    key = hash_bytes(&tile_cands, sizeof tile_cands, key);
+    key = hash_bytes(&n_win, sizeof n_win, key);
+    key = hash_bytes(win, sizeof(gb_window_t) * (size_t)n_win, key);
     ctx->clock++;
     for (auto& p : ctx->plans)
         if (p.key == key && p.prec == prec && p.n_win == n_win && p.tile_cands == tile_cands &&

@@ -83,3 +83,27 @@ def test_n_for_band_is_the_smallest_power_of_two():
         n = wk.n_for_band(f, T)
         bins = 2 * float(wk.bandwidth_max(f, T, 1.0)) * T
         assert n & (n - 1) == 0 and n >= 32 and n >= bins and (n == 32 or n / 2 < bins)
+
+
+def test_layouts_are_kept_by_value():
+    """The binding's window layouts: equal rows share one, changed or unhashable rows are converted anew, and
+    only gapless candidate ranges count as covering the rows."""
+    from paper_2307_03763_gb300 import api
+    ctx = api.Context.__new__(api.Context)
+    ctx._layouts = {}
+    rows = [(5, 32, 32, 0, 0, 3), (9, 32, 64, 32, 3, 4)]
+    lay = ctx._layout(rows)
+    assert lay is ctx._layout([tuple(r) for r in rows]) and lay is ctx._layout(tuple(rows))
+    assert lay is ctx._layout([list(r) for r in rows]) and lay is ctx._layout(np.array(rows))
+    assert lay is ctx._layout([tuple(float(x) for x in r) for r in rows])
+    assert (lay.n, lay.covered, lay.kmax) == (2, 7, 4)
+    assert [lay.arr[1].k0, lay.arr[1].W, lay.arr[1].N, lay.arr[1].data_off, lay.arr[1].cand_off,
+            lay.arr[1].n_cand] == [9, 32, 64, 32, 3, 4]
+    grown = np.array(rows)
+    grown[1, 5] = 6
+    assert ctx._layout(grown).kmax == 6 and ctx._layout(rows) is lay
+    scalars = [tuple(np.int64(x) for x in r) for r in rows]
+    assert ctx._layout(scalars) is lay
+    assert ctx._layout([(5, 32, 32, 0, 0, 3), (9, 32, 64, 32, 4, 4)]).covered == -1
+    assert ctx._layout([(5, 32, 32, 0, 0, 3), (9, 32, 64, 32, 2, 4)]).covered == -1
+    assert ctx._layout([]).covered == 0
