@@ -142,10 +142,11 @@ int gb_loglik_grad_aet(gb_ctx_t* ctx, int prec, const gb_window_t* win, int32_t 
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_error(ctx, e, "gb_loglik_grad: cudaSetDevice");
     const Plan* plan = nullptr;
-    // distinct plan keys for the gradient kernels; FP64: CTAs of two warps;
-    // mixed: warp work items of at most 32 candidates
+    // distinct plan keys for the gradient kernels; FP64: CTAs of two warps, at
+    // most 8 candidates each (32,768 candidates at N = 256: 4.77 ms; 4 or 16
+    // each: 4.95 and 5.36 ms); mixed: warp work items of at most 32 candidates
     int item = (int)std::min<int64_t>(32, std::max<int64_t>(1, (total + sm_count(ctx) * 8 - 1) / (sm_count(ctx) * 8)));
-    rc = get_plan(ctx, prec + 16, win, n_win, prec == GB_MIXED ? item : tile_size(ctx, total, 2), &plan);
+    rc = get_plan(ctx, prec + 16, win, n_win, prec == GB_MIXED ? item : std::min(tile_size(ctx, total, 2), 16), &plan);
     if (rc != GB_OK) return rc;
     if (prec == GB_FP64)
         return launch_grad_fp64(ctx, *plan, dA, dE, wA, wE, theta, logL, grad, dT, wT, (cudaStream_t)stream);

@@ -363,6 +363,13 @@ int get_plan(gb_ctx* ctx, int prec, const gb_window_t* win, int32_t n_win, int t
         split_last(sorted, (size_t)sms * 3 / 2);
         split_last(sorted, (size_t)sms * 3 / 4);
     }
+    if (prec == GB_FP64 + 16 && tile_cands >= 8) {   // the gradient's: four CTAs per SM
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms <= 0)
+            sms = 152;
+        split_last(sorted, (size_t)sms * 2);
+        split_last(sorted, (size_t)sms);
+    }
 
     Plan p;
     p.key = key;

@@ -209,12 +209,23 @@ struct GeoFx {
     Bx n0x, n0y, n0z, n1x, n1y, n1z, ca, sa;
 };
 
-// Slow part of sample n of N = 2^lg: A, E (and T with T3) as integers, whose
-// transforms times c.sA, c.sE, c.sT are the channels' bin values.
-// krho_q30: (L/c)/(3 1024 s) in Q30.
-template <int TIER, bool T3>
-GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q30, int n, int lg, int sh, fx (&o)[6]) {
-    const int u = n << (31 - lg);   // n/N in Q31
+// What a sample's response is made of, before the links are combined.
+struct MidFx {
+    int u;                     // n/N in Q31
+    fx a, b[3];                // a and b = a k.n of the arms, Q62
+    fx kn[3];                  // k.n, Q60
+    fx nu[3], nv[3];           // n.u, n.v, Q62
+    fx K;                      // K / 512 s, Q60
+    uint64_t ph;               // carrier phase, 2^-64 cycles
+    int ep[3];                 // eps of the receivers, Q57
+    fx co[3], si[3];           // exp(i theta) of the arms, Q62
+    Bx C1, S1;                 // amplitude polynomials, Q62
+};
+
+// krho_q30: (L/c)/(3 1024 s) in Q30
+template <int TIER>
+GB_FX void middle_fx(const CandFx& c, const GeoFx& g, int krho_q30, int n, int lg, MidFx& m) {
+    const int u = m.u = n << (31 - lg);
     // projections of the arms; the third arm closes the triangle
     Dot d = mul(c.k0, g.n0x);
     d.add(c.k1, g.n0y);
@@ -225,17 +236,20 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
     d.add(c.k2, g.n1z);
     const fx kn1 = d.get();
     const fx kn2 = -kn0 - kn1;
+    m.kn[0] = kn0;
+    m.kn[1] = kn1;
+    m.kn[2] = kn2;
     // a, b = a k.n in Q62
-    const fx a = c.a0 + (mulu(c.a1, u).get() >> 7);
+    const fx a = m.a = c.a0 + (mulu(c.a1, u).get() >> 7);
     const Bx ab = bal(a);
-    fx b[3];
+    fx* b = m.b;
     b[0] = mul(ab, bal(kn0)).get<4>();
     b[1] = mul(ab, bal(kn1)).get<4>();
     b[2] = -b[0] - b[1];
     // carrier phase, 2^-64 cycles: polynomial, Doppler f0 K, -fdot T u K + fdot K^2/2
     d = mul(c.Kc, g.ca);
     d.add(c.Ks, g.sa);
-    const fx K = d.get();   // Q60, K / 512 s
+    const fx K = m.K = d.get();
     const Bx Kb = bal(K);
     uint64_t ph = c.C0 + c.D1 * (uint64_t)(unsigned)n;
     {
@@ -248,6 +262,7 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         const fx t = (mulu(c.w1, u).get() >> 1) - mul(c.w2, Kb).get();   // Q60
         ph -= (uint64_t)mul(bal(t), Kb).get<8>();
     }
+    m.ph = ph;
     // eps of the three receivers in Q57 (see the head of the file); k.rho_j in
     // units of (L/c)/3 s: the differences of the arms' k.n
     int ep0, ep1, ep2;
@@ -261,6 +276,9 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         ep1 = (int)(wide(t1, c.FD) >> 30);
         ep2 = (int)(wide(t2, c.FD) >> 30);
     }
+    m.ep[0] = ep0;
+    m.ep[1] = ep1;
+    m.ep[2] = ep2;
     // arm phase factors; z = 3 theta + 3 (eps_i + eps_j)/2
     fx c0, s0, c1, s1, c2, s2;
     cis_third<TIER>(b[1] - b[2] + 48ll * (ep0 + ep1), c0, s0);   // Q57 -> Q62 and 3/2: x 48
@@ -278,22 +296,27 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         c2 -= cr;
         s2 += sr;
     }
+    m.co[0] = c0;
+    m.co[1] = c1;
+    m.co[2] = c2;
+    m.si[0] = s0;
+    m.si[1] = s1;
+    m.si[2] = s2;
     // amplitude polynomials C1 = a sin 2a cos a / (a0 sin 2a0), S1 = a sin 2a sin a / (a0 sin 2a0)
-    Bx C1, S1;
     {
         int r = c.cc4 + (int)(wide(c.cc5, u) >> 31);
         r = c.cc3 + (int)(wide(r, u) >> 31);
         fx q = c.cc2 + (wide(r, u) >> 22);
         q = c.cc1 + mulu(bal(q), u).get();   // Q64 -> Q63 -> Q62
-        C1 = bal(c.cc0 + mulu(bal(q), u).get());
+        m.C1 = bal(c.cc0 + mulu(bal(q), u).get());
         r = c.cs4 + (int)(wide(c.cs5, u) >> 31);
         r = c.cs3 + (int)(wide(r, u) >> 31);
         q = c.cs2 + (wide(r, u) >> 22);
         q = c.cs1 + mulu(bal(q), u).get();
-        S1 = bal(c.cs0 + mulu(bal(q), u).get());
+        m.S1 = bal(c.cs0 + mulu(bal(q), u).get());
     }
     // n.u, n.v in Q62
-    fx nu[3], nv[3];
+    fx *nu = m.nu, *nv = m.nv;
     d = mul(c.u0, g.n0x);
     d.add(c.u1, g.n0y);
     d.add(c.u2, g.n0z);
@@ -310,20 +333,44 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
     d.add(c.v1, g.n1y);
     nv[1] = d.get<2>();
     nv[2] = -nv[0] - nv[1];
+}
+
+// polarisation response of arm k: G = n.H.n at unit amplitude, Q60, and
+// F+ = (n.u)^2 - (n.v)^2, Fx/2 = (n.u)(n.v), Q60
+struct PolFx {
+    Bx Fp, Fx;
+    fx Gr, Gi;
+};
+GB_FX PolFx pol_fx(const CandFx& c, const MidFx& m, int k) {
+    PolFx p;
+    p.Fp = bal(mul(bal(m.nu[k] - m.nv[k]), bal(m.nu[k] + m.nv[k])).get());
+    p.Fx = bal(mul(bal(m.nu[k]), bal(m.nv[k])).get());
+    Dot gr = mul(c.gpr, p.Fp), gi = mul(c.gpi, p.Fp);
+    gr.add(c.gxr, p.Fx);
+    gi.add(c.gxi, p.Fx);
+    p.Gr = gr.get<4>();
+    p.Gi = gi.get<4>();
+    return p;
+}
+
+// Slow part of sample n of N = 2^lg: A, E (and T with T3) as integers, whose
+// transforms times c.sA, c.sE, c.sT are the channels' bin values.
+template <int TIER, bool T3>
+GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q30, int n, int lg, int sh, fx (&o)[6]) {
+    MidFx m;
+    middle_fx<TIER>(c, g, krho_q30, n, lg, m);
+    const Bx C1 = m.C1, S1 = m.S1;
+    const fx a = m.a;
+    const fx* b = m.b;
     Dot Ar{0, 0}, Ai{0, 0}, Er{0, 0}, Ei{0, 0}, Tr{0, 0}, Ti{0, 0};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         // polarisation response times the arm's phase factor: H in Q58
-        const Bx Fp = bal(mul(bal(nu[k] - nv[k]), bal(nu[k] + nv[k])).get());   // Q60
-        const Bx Fx = bal(mul(bal(nu[k]), bal(nv[k])).get());
-        Dot gr = mul(c.gpr, Fp), gi = mul(c.gpi, Fp);
-        gr.add(c.gxr, Fx);
-        gi.add(c.gxi, Fx);
-        const fx Gi_ = gi.get<4>();
-        const Bx Gr = bal(gr.get<4>()), Gi = bal(Gi_);   // Q60
-        const Bx ck = bal(k == 0 ? c0 : k == 1 ? c1 : c2), sk = bal(k == 0 ? s0 : k == 1 ? s1 : s2);
+        const PolFx G = pol_fx(c, m, k);
+        const Bx Gr = bal(G.Gr), Gi = bal(G.Gi);
+        const Bx ck = bal(m.co[k]), sk = bal(m.si[k]);
         Dot hr = mul(Gr, ck), hi = mul(Gr, sk);
-        hr.add(bal(-Gi_), sk);
+        hr.add(bal(-G.Gi), sk);
         hi.add(Gi, ck);
         const fx Hi_ = hi.get();   // Q58
         const Bx Hr = bal(hr.get()), Hi = bal(Hi_), mHi = bal(-Hi_);
@@ -334,7 +381,7 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         const Bx Sh = bal(sp + sm), Dh = bal(sp - sm);
         const fx p = mul(Sh, C1).get(), q = mul(Dh, S1).get();
         // dp = Sh S1 Delta/2, dq = Dh C1 Delta/2 in Q58, Delta = eps of the + receiver - eps of the - one
-        const int dl = k == 0 ? ep1 - ep0 : k == 1 ? ep2 - ep1 : ep0 - ep2;   // Q57
+        const int dl = m.ep[k == 2 ? 0 : k + 1] - m.ep[k];   // Q57
         const int ss = (int)(wide(Sh.h, S1.h) >> 30), dc = (int)(wide(Dh.h, C1.h) >> 30);   // Q30
         const fx dp = (wide(ss, dl) >> 30) * 4, dq = (wide(dc, dl) >> 30) * 4;   // Q57 of value/2 = Q58; x 4: Q60
         // A sqrt2 = Z - X, E sqrt6 = X - 2Y + Z, T sqrt3 = X + Y + Z: coefficients of H_k
@@ -373,7 +420,7 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         }
     }
     fx co, si;
-    cis_table(ph, tw, co, si);
+    cis_table(m.ph, tw, co, si);
     const Bx cb = bal(co), sb = bal(si), msb = bal(-si);
     {
         const Bx r = bal(Ar.get()), i = bal(Ai.get());   // Q54
@@ -420,6 +467,32 @@ struct FxTrig {
     double sb, cb, sl, cl, s2, c2, ci, sa, ca;   // of beta, lambda, 2 psi, iota, a0 = pi f0 L/c
 };
 
+// Taylor coefficients in v, a = a0 (1 + v), of
+//   C1 = a sin 2a cos a/(a0 sin 2a0) = (1 + v) (sin 3a + sin a)/(2 sin 2a0),
+//   S1 = a sin 2a sin a/(a0 sin 2a0) = (1 + v) (cos a - cos 3a)/(2 sin 2a0),
+// from sin a0 and cos a0
+GB_FX void amplitude_series(double a0, double s1, double c1, double (&Cv)[6], double (&Sv)[6]) {
+    const double s3 = s1 * (3.0 - 4.0 * s1 * s1), c3 = c1 * (4.0 * c1 * c1 - 3.0);
+    const double inv = 0.25 / (s1 * c1);
+    double C[6], S[6];
+    double ak = 1.0, p3 = 1.0;   // a0^k/k!, 3^k
+    for (int k = 0; k < 6; ++k) {
+        const int m = k & 3;
+        const double ds3 = m == 0 ? s3 : m == 1 ? c3 : m == 2 ? -s3 : -c3, ds1 = m == 0 ? s1 : m == 1 ? c1 : m == 2 ? -s1 : -c1;
+        const double dc3 = m == 0 ? c3 : m == 1 ? -s3 : m == 2 ? -c3 : s3, dc1 = m == 0 ? c1 : m == 1 ? -s1 : m == 2 ? -c1 : s1;
+        C[k] = (p3 * ds3 + ds1) * ak * inv;
+        S[k] = (dc1 - p3 * dc3) * ak * inv;
+        ak *= a0 / (double)(k + 1);
+        p3 *= 3.0;
+    }
+    C[0] = c1;
+    S[0] = s1;
+    for (int k = 0; k < 6; ++k) {
+        Cv[k] = C[k] + (k > 0 ? C[k - 1] : 0.0);
+        Sv[k] = S[k] + (k > 0 ? S[k - 1] : 0.0);
+    }
+}
+
 // Candidate constants; c.tier = -1 when a parameter is outside the ranges.
 // arm_c = L/c; the caller supplies the sines and cosines.
 GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int lg, const FxTrig& t, CandFx& c) {
@@ -429,8 +502,12 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     const double a0 = pi * f0 * arm_c, a1 = pi * fd * T * arm_c, eta = fd * T / f0;
     const double xmax = 2.0 * fmax(fabs(a0), fabs(a0 + a1));
     const double r = 1.495978707e11 / 299792458.0;
-    const double Kc = -r * t.cb * t.cl, Ks = -r * t.cb * t.sl;
+    // f0 K reaches several cycles: its two products as double-word values
+    const double rc = -r * t.cb, rc_e = fma(-r, t.cb, -rc);
+    const double Kc = rc * t.cl, Ks = rc * t.sl;
     const double Fc = f0 * Kc, Fs = f0 * Ks;
+    const double Fc_e = fma(f0, Kc, -Fc) + f0 * (fma(rc, t.cl, -Kc) + rc_e * t.cl);
+    const double Fs_e = fma(f0, Ks, -Fs) + f0 * (fma(rc, t.sl, -Ks) + rc_e * t.sl);
     // fdot T^2/2 as a double-word value: it reaches hundreds of cycles
     const double fdT = fd * T, fdT_e = fma(fd, T, -fdT), c2h = 0.5 * (fdT * T),
                  c2l = 0.5 * (fma(fdT, T, -(fdT * T)) + fdT_e * T), c2r = rint(c2h);
@@ -456,8 +533,8 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     c.gxi = to_bx(-2.0 * (Ax * t.c2), 0x1p60);
     c.Kc = to_bx(Kc, 0x1p53);
     c.Ks = to_bx(Ks, 0x1p53);
-    c.Fc = to_bx(Fc, 0x1p57);
-    c.Fs = to_bx(Fs, 0x1p57);
+    c.Fc = bal(to_fx(Fc, 0x1p57) + to_fx(Fc_e, 0x1p57));
+    c.Fs = bal(to_fx(Fs, 0x1p57) + to_fx(Fs_e, 0x1p57));
     c.w1 = to_bx(w1, 0x1p62);
     c.w2 = to_bx(w2, 0x1p64);
     c.c2 = to_bx((c2h - c2r) + c2l, 0x1p62);
@@ -473,27 +550,12 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     const double dr = delta - N * rint(delta / N);
     const double sc = ldexp(1.0, 62 - lg);
     c.D1 = (uint64_t)to_fx(dr, sc) * 4u + (uint64_t)to_fx(-a1 * 0.63661977236758134, 4.0 * sc);
-    // C1(v) = (1 + v) (sin 3a + sin a)/(2 sin 2a0), S1(v) = (1 + v) (cos a - cos 3a)/(2 sin 2a0),
-    // a = a0 (1 + v), v = eta u: Taylor coefficients in u
-    const double s1 = t.sa, c1 = t.ca, s3 = s1 * (3.0 - 4.0 * s1 * s1), c3 = c1 * (4.0 * c1 * c1 - 3.0);
-    const double inv = 0.25 / (s1 * c1);
-    double C[6], S[6];
-    double ak = 1.0, p3 = 1.0;   // a0^k/k!, 3^k
-    for (int k = 0; k < 6; ++k) {
-        const int m = k & 3;
-        const double ds3 = m == 0 ? s3 : m == 1 ? c3 : m == 2 ? -s3 : -c3, ds1 = m == 0 ? s1 : m == 1 ? c1 : m == 2 ? -s1 : -c1;
-        const double dc3 = m == 0 ? c3 : m == 1 ? -s3 : m == 2 ? -c3 : s3, dc1 = m == 0 ? c1 : m == 1 ? -s1 : m == 2 ? -c1 : s1;
-        C[k] = (p3 * ds3 + ds1) * ak * inv;
-        S[k] = (dc1 - p3 * dc3) * ak * inv;
-        ak *= a0 / (double)(k + 1);
-        p3 *= 3.0;
-    }
-    C[0] = c1;
-    S[0] = s1;
+    double Cv[6], Sv[6];
+    amplitude_series(a0, t.sa, t.ca, Cv, Sv);
     double e = 1.0, Cu[6], Su[6];
     for (int k = 0; k < 6; ++k) {
-        Cu[k] = (C[k] + (k > 0 ? C[k - 1] : 0.0)) * e;
-        Su[k] = (S[k] + (k > 0 ? S[k - 1] : 0.0)) * e;
+        Cu[k] = Cv[k] * e;
+        Su[k] = Sv[k] * e;
         e *= eta;
     }
     c.cc0 = to_fx(Cu[0], 0x1p62);
@@ -511,7 +573,7 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     // |T| < 6 a^3 + 4 a 2^-20 (q < a^3/3, dp < a 2^-26): shifted up to A's range
     c.tsh = 0;
     for (double b = 6.0 * a0 * a0 * a0 * 1.01 + 0x1p-18 * a0; b < 3.0 && c.tsh < 24; b *= 2.0) ++c.tsh;
-    const double amp = A * (8.0 * a0 * s1 * c1) * (T / (2.0 * N)) * ldexp(1.0, fx_shift(lg) - 52);   // 4 a0 sin 2a0
+    const double amp = A * (8.0 * a0 * t.sa * t.ca) * (T / (2.0 * N)) * ldexp(1.0, fx_shift(lg) - 52);   // 4 a0 sin 2a0
     c.sA = amp * 0.70710678118654752;
     c.sE = amp * 0.40824829046386302;
     c.sT = amp * 0.57735026918962576 * ldexp(1.0, -c.tsh);

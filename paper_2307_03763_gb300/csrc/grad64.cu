@@ -1,13 +1,27 @@
-// grad64.cu -- gradient of the window log-likelihood, plain IEEE double.
+// grad64.cu -- gradient of the window log-likelihood, double precision.
 //
 // With h_k = (T/2N) S_m and r_m = w_k (d_k - h_k) on window bins (0 elsewhere),
 //   d logL / d theta_i = (4/T) sum_k w_k Re[(d_k - h_k) conj(d h_k/d theta_i)]
 //                      = (2/N) Re sum_n  conj(c_n) d s_n / d theta_i,
 //   c_n = conj(sum_m conj(r_m) exp(-2 pi i m n / N))   (the adjoint of the DFT).
-// Per candidate the kernel (1) computes the template, (2) forms the residual
-// r and logL, (3) runs the adjoint FFT to get c_n, and (4) sweeps the samples
-// in reverse mode: each sample's forward values (the fast/slow response of
-// Sec. II, in the same link form as the FP64 likelihood), then the adjoints
+// Per candidate one warp (1) computes the template, (2) forms the residual r
+// and logL, (3) runs the adjoint FFT to get c_n, and (4) sweeps the samples in
+// reverse mode.  The template, the adjoint FFT and the sweep run in 64-bit
+// fixed point (fx64.cuh, fx64_grad.cuh): the residual is scaled by a power of
+// two per candidate, the cotangents again before the sweep, and every sample
+// leaves 22 sums in double that are contracted with the candidate's constants
+// at the end, one candidate per lane.
+//
+// Measured on GB300, 64 windows x 512 candidates at N = 256: 33.8 ms with every
+// step in double (FP64 pipe 84% busy), 4.8 ms in this form (8,900 warp
+// instructions per 32 samples, the multiply pipe 54-65% and the FP64 pipe 35%
+// busy with eight warps per SM, the most that 255 registers leave).  Error of the
+// gradients against 113-bit arithmetic: 1e-15 ... 8e-15 of their norm per
+// parameter, where the double form had 3e-15 ... 5e-14.
+//
+// Candidates outside the fixed-point ranges take the plain double form: each
+// sample's forward values (the fast/slow response of
+// Sec. II, in the same link form as the likelihood's), then the adjoints
 // of the channel samples c_n propagated back through the TDI combination,
 // the six links and the three receiver phases to the parameters.  The
 // amplitude, inclination and polarisation enter only through the two complex
@@ -24,25 +38,20 @@
 //   dv/dlambda = (cos lambda, sin lambda, 0),
 //   d/dX [sinc(X) e^{-iX}] from the derivative of its series (or, evaluated
 //   directly, (e^{-2iX} - sinc(X) e^{-iX}) / X).
-#include <cmath>
-
-#include "gb_internal.cuh"
+#include "fp64_common.cuh"
+#include "fx64_grad.cuh"
 
 namespace gb {
 namespace {
 
 constexpr int kWarpsG = 2;
+constexpr int kSumsG = kGSums + 4;   // sums a candidate leaves for its contraction: adjoint_fx's, <d|h>, <h|h>, norm
+constexpr int kCapG = 16;   // candidates a warp sets up at a time
 constexpr int K = 8;   // f0, fdot, beta, lambda, A, iota, psi, phi0
 
-struct C {
-    double x, y;
-};
-__device__ __forceinline__ C cadd(C a, C b) { return {a.x + b.x, a.y + b.y}; }
-__device__ __forceinline__ C csub(C a, C b) { return {a.x - b.x, a.y - b.y}; }
-__device__ __forceinline__ C cmul(C a, C b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+using C = C64;
 // a conj(b)
 __device__ __forceinline__ C cmulc(C a, C b) { return {a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y}; }
-__device__ __forceinline__ C cscale(C a, double s) { return {a.x * s, a.y * s}; }
 // Re(conj(a) b)
 __device__ __forceinline__ double redot(C a, C b) { return a.x * b.x + a.y * b.y; }
 
@@ -79,21 +88,26 @@ struct CandG {
     C al, ga, al_i[3], ga_i[3];      // alpha, gamma and their derivatives wrt A, iota, psi
     double f0, fd, delta, phi0c;
     double D0r, D0i, eps;            // exp(-i f0/f*), fdot/f*
-    long long q;
-    int bad, J;
+    int J;
 };
 
-__device__ void setup_grad(const double* th, double T, double inv_fstar, CandG& c) {
+// One candidate: its template's constants, and what the gradient adds to the
+// fixed-point form, or the plain double form's constants.
+struct CandGT {
+    CandT t;
+    union {
+        struct {
+            CandGFx g;
+            FinGFx fin;
+        };
+        CandG d;
+    };
+};
+
+__device__ void setup_grad(const double* th, double T, double inv_fstar, double delta, CandG& c) {
     const double f0 = th[0], fd = th[1], beta = th[2], lam = th[3];
     const double A = th[4], iota = th[5], psi = th[6], phi0 = th[7];
-    bool bad = false;
-    for (int i = 0; i < 8; ++i) bad |= !isfinite(th[i]);
-    c.bad = bad;
-    const double f0T = __dmul_rn(f0, T);
-    const double xm = __dadd_rn(f0T, __dmul_rn(__dmul_rn(__dmul_rn(0.5, fd), T), T));
-    const double qd = floor(__dadd_rn(xm, 0.5));
-    c.q = bad ? 0 : (long long)qd;
-    c.delta = __dadd_rn(f0T, -qd);
+    c.delta = delta;
     c.f0 = f0;
     c.fd = fd;
     c.phi0c = phi0 * 0.15915494309189535;   // 1 / (2 pi)
@@ -172,10 +186,7 @@ __device__ __forceinline__ void transfer(double X, int J, C& V, C& Vd) {
     if (DER) Vd = {X * dre, dim};
 }
 
-struct Geo {
-    double T, T_over_N, inv_fstar, scale;
-    int N, logN;
-};
+using Geo = Geo64;
 
 // Forward values of one sample (Sec. II): receiver phasors, the six links
 // z_ij = -i a V(a (1 -+ k.n)) (n.H.n) exp(2 pi i cyc), D = exp(-i f/f*) and
@@ -398,27 +409,224 @@ __device__ void fft_inplace(int N, int logN, const C* tw, C* bufA, C* bufE, C* b
     }
 }
 
-__device__ __forceinline__ double wsum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// Gradient of one plain-double candidate (one warp); lane 0 writes row `row`.
+__device__ __noinline__ void grad_plain(const CandG& c, long long q, int64_t row, const Geo& g, const OrbitTables64& tab,
+                                        const C* tw, C* bufA, C* bufE, C* bufT, const gb_window_t& win, double dd,
+                                        const C* __restrict__ dA, const C* __restrict__ dE,
+                                        const double* __restrict__ wA, const double* __restrict__ wE,
+                                        const C* __restrict__ dT, const double* __restrict__ wT,
+                                        double* __restrict__ logL_out, double* __restrict__ grad_out, int lane) {
+    const int N = g.N;
+    const double T = g.T;
+    const bool useT = bufT != nullptr;
+    // (1) template
+    template_value(c, g, tab, bufA, bufE, bufT, lane);
+    fft_inplace(N, g.logN, tw, bufA, bufE, bufT, lane);
+    // (2) logL and residual r_m = w (d - h) at DFT index m mod N, in place
+    double sdh = 0.0, shh = 0.0;
+    for (int idx = lane; idx < N; idx += 32) {
+        const int m = idx < N / 2 ? idx : idx - N;      // signed frequency offset
+        const int64_t kk = q + m - win.k0;
+        const C hA = cscale(bufA[idx], g.scale), hE = cscale(bufE[idx], g.scale);
+        C rA = {0.0, 0.0}, rE = {0.0, 0.0};
+        if (kk >= 0 && kk < win.W) {
+            const C a = dA[win.data_off + kk], e = dE[win.data_off + kk];
+            const double wa = wA[win.data_off + kk], we = wE[win.data_off + kk];
+            sdh += wa * (a.x * hA.x + a.y * hA.y) + we * (e.x * hE.x + e.y * hE.y);
+            shh += wa * (hA.x * hA.x + hA.y * hA.y) + we * (hE.x * hE.x + hE.y * hE.y);
+            rA = {wa * (a.x - hA.x), wa * (a.y - hA.y)};
+            rE = {we * (e.x - hE.x), we * (e.y - hE.y)};
+        }
+        // conjugate for the adjoint transform: c = conj(FFT(conj(r)))
+        bufA[idx] = {rA.x, -rA.y};
+        bufE[idx] = {rE.x, -rE.y};
+        if (useT) {
+            const C hT = cscale(bufT[idx], g.scale);
+            C rT = {0.0, 0.0};
+            if (kk >= 0 && kk < win.W) {
+                const C t = dT[win.data_off + kk];
+                const double wt = wT[win.data_off + kk];
+                sdh += wt * (t.x * hT.x + t.y * hT.y);
+                shh += wt * (hT.x * hT.x + hT.y * hT.y);
+                rT = {wt * (t.x - hT.x), wt * (t.y - hT.y)};
+            }
+            bufT[idx] = {rT.x, -rT.y};
+        }
+    }
+    sdh = warp_sum(sdh) * (4.0 / T);
+    shh = warp_sum(shh) * (4.0 / T);
+    __syncwarp();
+    // (3) bit-reversal permutation in place, then the same forward FFT
+    for (int i = lane; i < N; i += 32) {
+        const int j = (int)(__brev((unsigned)i) >> (32 - g.logN));
+        if (i < j) {
+            const C ta = bufA[i];
+            bufA[i] = bufA[j];
+            bufA[j] = ta;
+            const C te = bufE[i];
+            bufE[i] = bufE[j];
+            bufE[j] = te;
+            if (useT) {
+                const C tt = bufT[i];
+                bufT[i] = bufT[j];
+                bufT[j] = tt;
+            }
+        }
+    }
+    __syncwarp();
+    fft_inplace(N, g.logN, tw, bufA, bufE, bufT, lane);
+    // (4) reverse-mode sweep: the adjoint of sample n is c_n = conj(buf[n])
+    Acc acc = {0.0, 0.0, 0.0, 0.0, 0.0, {0.0, 0.0}, {0.0, 0.0}};
+    for (int n = lane; n < N; n += 32) {
+        const C cA = {bufA[n].x, -bufA[n].y}, cE = {bufE[n].x, -bufE[n].y};
+        const C cT = useT ? C{bufT[n].x, -bufT[n].y} : C{0.0, 0.0};
+        sample_adjoint(c, g, tab, n, cA, cE, cT, useT, acc);
+    }
+    double gacc[K];
+    gacc[0] = acc.f0;
+    gacc[1] = acc.fd;
+    gacc[2] = acc.beta;
+    gacc[3] = acc.lam;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gacc[4 + k] = redot(acc.al, c.al_i[k]) + redot(acc.ga, c.ga_i[k]);
+    gacc[7] = acc.phi0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) gacc[k] = warp_sum(gacc[k]) * (2.0 / (double)N);
+    if (lane == 0) {
+        if (logL_out) logL_out[row] = sdh - 0.5 * shh - 0.5 * dd;
+#pragma unroll
+        for (int k = 0; k < K; ++k) grad_out[8 * row + k] = gacc[k];
+    }
+    __syncwarp();
 }
 
-__global__ void __launch_bounds__(kWarpsG * 32) grad64_kernel(
+// Bits of |x|'s high word, and the largest of them over a warp: the exponent
+// of the largest cotangent without an FP64 compare
+__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7FFFFFFFu; }
+
+// Residual, adjoint transform and sweep of one candidate in fixed point (one
+// warp), its template's bin values in buf.  Leaves adjoint_fx's sums in out,
+// then <d|h> and <h|h> (before 4/T) and the value of a unit of the cotangents
+// (NaN when the data are not finite).
+template <int TIER, bool T3>
+__device__ __noinline__ void sweep_fx(const CandGT& c, const Geo& g, const FxTab& ft, C* buf, int stride, const gb_window_t& win,
+                           const C* __restrict__ dA, const C* __restrict__ dE, const double* __restrict__ wA,
+                           const double* __restrict__ wE, const C* __restrict__ dT, const double* __restrict__ wT,
+                           int lane, double* out) {
+    const int N = g.N, lg = g.logN;
+    constexpr int NCH = T3 ? 3 : 2;
+    double sdh = 0.0, shh = 0.0;
+    unsigned top = 0;
+    // conj(r), r = w (d - h), in place at its DFT index
+    for (int idx = lane; idx < N; idx += 32) {
+        const int m = idx < N / 2 ? idx : idx - N;      // signed frequency offset
+        const int64_t kk = c.t.q + m - win.k0;
+        const bool in = kk >= 0 && kk < win.W;
+        const int e = sw(idx);
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            C r = {0.0, 0.0};
+            if (in) {
+                const C h = buf[ch * stride + e], d = (ch == 0 ? dA : ch == 1 ? dE : dT)[win.data_off + kk];
+                const double w = (ch == 0 ? wA : ch == 1 ? wE : wT)[win.data_off + kk];
+                sdh += w * (d.x * h.x + d.y * h.y);
+                shh += w * (h.x * h.x + h.y * h.y);
+                r = {w * (d.x - h.x), -(w * (d.y - h.y))};
+                top = max(top, max(abs_hi(r.x), abs_hi(r.y)));
+            }
+            buf[ch * stride + e] = r;
+        }
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    __syncwarp();
+    // to integers below 2^(61 - lg), A's normalisation for every channel, and
+    // into bit-reversed order
+    const int k = min(1000, 61 - lg - ((int)(top >> 20) - 1022));
+    const double s0 = scalbn(1.0, k);
+    const double sc[3] = {s0, s0 * 0.57735026918962576, s0 * 0.81649658092772603};
+    Z64* z = (Z64*)buf;
+    for (int i = lane; i < N; i += 32) {
+        const int j = (int)(__brev((unsigned)i) >> (32 - lg));
+        if (i > j) continue;
+        const int ei = sw(i), ej = sw(j);
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            const C a = buf[ch * stride + ei], b = buf[ch * stride + ej];
+            z[ch * stride + ej] = {__double2ll_rn(a.x * sc[ch]), __double2ll_rn(a.y * sc[ch])};
+            z[ch * stride + ei] = {__double2ll_rn(b.x * sc[ch]), __double2ll_rn(b.y * sc[ch])};
+        }
+    }
+    __syncwarp();
+    fft_fx<32, true>(z, stride, NCH, lg, ft.tw, sc, lane);
+    // normalise: the largest component into [2^59, 2^60)
+    unsigned big = 0;
+    for (int n = lane; n < N; n += 32) {
+        const int e = sw(n);
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            const Z64 v = z[ch * stride + e];
+            const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
+            big = max(big, (unsigned)max(x ^ (x >> 31), y ^ (y >> 31)));
+        }
+    }
+    big = __reduce_max_sync(0xffffffffu, big);
+    const int up = __clz(big) - 4;   // left shift, or right when negative
+    double acc[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc[j] = 0.0;
+    double(&sums)[kGSums] = *(double(*)[kGSums])acc;
+    for (int n = lane; n < N; n += 32) {
+        const int e = sw(n);
+        fx gr[3], gi[3];
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            const Z64 v = z[ch * stride + e];
+            gr[ch] = up >= 0 ? v.x << up : v.x >> -up;
+            gi[ch] = up >= 0 ? v.y << up : v.y >> -up;
+        }
+        const int4 a = __ldg(ft.geo + n), b = __ldg(ft.geo + N + n), f = __ldg(ft.geo + 2 * N + n),
+                   h = __ldg(ft.geo + 3 * N + n);
+        const GeoFx ge{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}, {f.x, f.y}, {f.z, f.w}, {h.x, h.y}, {h.z, h.w}};
+        adjoint_fx<TIER, T3>(c.t.f, c.g, ge, ft.tw, g.krho_q30, n, lg, gr, gi, sums);
+    }
+    acc[kGSums] = sdh;
+    acc[kGSums + 1] = shh;
+    // warp sums by halves: lane j ends with the total of value j
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const double keep = upper ? acc[j + o] : acc[j], send = upper ? acc[j] : acc[j + o];
+            acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    if (lane < kGSums + 2) out[lane] = acc[0];
+    if (lane == 31) out[kGSums + 2] = top >= 0x7FF00000u ? nan("") : scalbn(1.0, 60 - k - up);
+    __syncwarp();
+}
+
+// Resident CTAs per SM, of two warps at 255 registers (five or six at fewer
+// registers: 24% slower, from spills in the sweep).
+constexpr int kMinCtasG = 4;
+
+__global__ void __launch_bounds__(kWarpsG * 32, kMinCtasG) grad64_kernel(
     const gb_window_t* __restrict__ wins, const Tile* __restrict__ tiles, TabSet64 tabs, const C* __restrict__ tw_g,
-    double T, double fstar, const C* __restrict__ dA, const C* __restrict__ dE, const double* __restrict__ wA,
-    const double* __restrict__ wE, const double* __restrict__ theta, double* __restrict__ logL_out,
-    double* __restrict__ grad_out, const C* __restrict__ dT, const double* __restrict__ wT, int* status,
-    int n_max) {
+    TabSetFx fxt, double T, double fstar, const C* __restrict__ dA, const C* __restrict__ dE,
+    const double* __restrict__ wA, const double* __restrict__ wE, const double* __restrict__ theta,
+    double* __restrict__ logL_out, double* __restrict__ grad_out, const C* __restrict__ dT,
+    const double* __restrict__ wT, int* status, int n_max) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = (C*)smem_raw;
-    double* red = (double*)(tw + kTwiddles);
-    CandG* cands = (CandG*)(red + kWarpsG);
-    C* bufs = (C*)(cands + kWarpsG * 32);
+    FxTw* tw = (FxTw*)smem_raw;                                  // kTwiddles
+    double* red = (double*)(tw + kTwiddles);                     // kWarpsG
+    CandGT* cands = (CandGT*)(red + kWarpsG);                    // kWarpsG * kCapG
+    double* sums = (double*)(cands + kWarpsG * kCapG);           // kWarpsG * kCapG * kSumsG
+    C* bufs = (C*)(sums + kWarpsG * kCapG * kSumsG);             // kWarpsG * (2 or 3) * n_max
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Tile tile = tiles[blockIdx.x];
     const gb_window_t win = wins[tile.win];
-    for (int i = threadIdx.x; i < kTwiddles; i += blockDim.x) tw[i] = tw_g[i];
+    load_twiddles(fxt.tw, tw);
     // T enters windows whose lowest frequency is at least f*/2 (dT given)
     const bool useT = dT != nullptr && (double)win.k0 / T >= 0.5 * fstar;
     double acc = 0.0;
@@ -430,120 +638,72 @@ __global__ void __launch_bounds__(kWarpsG * 32) grad64_kernel(
             acc += wT[win.data_off + i] * (t.x * t.x + t.y * t.y);
         }
     }
-    acc = wsum(acc);
+    acc = warp_sum(acc);
     if (lane == 0) red[warp] = acc;
     __syncthreads();
     double dd = 0.0;
     for (int w = 0; w < kWarpsG; ++w) dd += red[w];
     dd *= 4.0 / T;
 
-    Geo g;
-    g.N = win.N;
-    g.logN = 31 - __clz(win.N);
-    g.T = T;
-    g.T_over_N = T / (double)win.N;
-    g.inv_fstar = 1.0 / fstar;
-    g.scale = T / (2.0 * (double)win.N);
+    const Geo g = geometry64(win.N, T, fstar, fxt.arm_c, fxt.krho_q30);
     const OrbitTables64 tab = tabs.t[g.logN - 5];
-    const int N = g.N;
-    C* bufA = bufs + (size_t)warp * (dT ? 3 : 2) * n_max;
-    C* bufE = bufA + n_max;
-    C* bufT = useT ? bufE + n_max : nullptr;
-    CandG* mycand = cands + warp * 32;
+    const FxTab ft{fxt.geo[g.logN - 5], tw, tw_g};
+    C* buf = bufs + (size_t)warp * (dT ? 3 : 2) * n_max;
+    CandGT* mycand = cands + warp * kCapG;
+    double* mysum = sums + warp * kCapG * kSumsG;
     const int64_t tlen = tile.c_end - tile.c_begin;
     const int64_t grp = (tlen + kWarpsG - 1) / kWarpsG;
     const int64_t c_lo = tile.c_begin + (int64_t)warp * grp;
     const int64_t c_hi = min(tile.c_end, c_lo + grp);
-    if (c_lo >= c_hi) return;
-    if (c_lo + lane < c_hi) setup_grad(theta + 8 * (c_lo + lane), T, g.inv_fstar, mycand[lane]);
-    __syncwarp();
-    for (int64_t cidx = c_lo; cidx < c_hi; ++cidx) {
-        const CandG& c = mycand[cidx - c_lo];
-        if (c.bad) {
-            if (lane == 0) {
-                if (logL_out) logL_out[cidx] = nan("");
-                for (int k = 0; k < K; ++k) grad_out[8 * cidx + k] = nan("");
+    for (int64_t c0 = c_lo; c0 < c_hi; c0 += kCapG) {
+        const int cnt = (int)min((int64_t)kCapG, c_hi - c0);
+        if (lane < cnt) {
+            CandGT& c = mycand[lane];
+            const double* th = theta + 8 * (c0 + lane);
+            FxTrig t;
+            double si;
+            setup_lane(th, g, c.t, t, si);
+            if (c.t.tier >= 0 && !setup_gfx(th, T, g.arm_c, t, c.g)) c.t.tier = -1;
+            if (c.t.tier >= 0) {
+                setup_fin(th, T, g.arm_c, g.logN, t, si, c.fin);
+            } else if (!c.t.bad) {
+                setup_grad(th, T, g.inv_fstar, __dadd_rn(__dmul_rn(th[0], T), -(double)c.t.q), c.d);
+            }
+        }
+        __syncwarp();
+        for (int i = 0; i < cnt; ++i) {
+            const CandGT& c = mycand[i];
+            if (c.t.bad) continue;
+            if (c.t.tier < 0) {
+                grad_plain(c.d, c.t.q, c0 + i, g, tab, tw_g, buf, buf + n_max, useT ? buf + 2 * n_max : nullptr, win,
+                           dd, dA, dE, wA, wE, dT, wT, logL_out, grad_out, lane);
+                continue;
+            }
+            template_any<32>(c.t, g, tab, ft, buf, n_max, useT, lane);
+            double* s = mysum + i * kSumsG;
+            if (c.t.tier == 0) {
+                if (useT) sweep_fx<0, true>(c, g, ft, buf, n_max, win, dA, dE, wA, wE, dT, wT, lane, s);
+                else sweep_fx<0, false>(c, g, ft, buf, n_max, win, dA, dE, wA, wE, dT, wT, lane, s);
+            } else {
+                if (useT) sweep_fx<1, true>(c, g, ft, buf, n_max, win, dA, dE, wA, wE, dT, wT, lane, s);
+                else sweep_fx<1, false>(c, g, ft, buf, n_max, win, dA, dE, wA, wE, dT, wT, lane, s);
+            }
+        }
+        // the sums' contraction, one candidate per lane
+        if (lane < cnt) {
+            const CandGT& c = mycand[lane];
+            const int64_t row = c0 + lane;
+            if (c.t.bad) {
+                if (logL_out) logL_out[row] = nan("");
+                for (int k = 0; k < K; ++k) grad_out[8 * row + k] = nan("");
                 atomicOr(status, kStatusNonFinite);
+            } else if (c.t.tier >= 0) {
+                const double* s = mysum + lane * kSumsG;
+                double gout[K];
+                finish_gfx(c.fin, T, s, s[kGSums + 2], gout);
+                if (logL_out) logL_out[row] = s[kGSums] * (4.0 / T) - 0.5 * (s[kGSums + 1] * (4.0 / T)) - 0.5 * dd;
+                for (int k = 0; k < K; ++k) grad_out[8 * row + k] = gout[k];
             }
-            continue;
-        }
-        // (1) template
-        template_value(c, g, tab, bufA, bufE, bufT, lane);
-        fft_inplace(N, g.logN, tw, bufA, bufE, bufT, lane);
-        // (2) logL and residual r_m = w (d - h) at DFT index m mod N, in place
-        double sdh = 0.0, shh = 0.0;
-        for (int idx = lane; idx < N; idx += 32) {
-            const int m = idx < N / 2 ? idx : idx - N;      // signed frequency offset
-            const int64_t kk = c.q + m - win.k0;
-            const C hA = cscale(bufA[idx], g.scale), hE = cscale(bufE[idx], g.scale);
-            C rA = {0.0, 0.0}, rE = {0.0, 0.0};
-            if (kk >= 0 && kk < win.W) {
-                const C a = dA[win.data_off + kk], e = dE[win.data_off + kk];
-                const double wa = wA[win.data_off + kk], we = wE[win.data_off + kk];
-                sdh += wa * (a.x * hA.x + a.y * hA.y) + we * (e.x * hE.x + e.y * hE.y);
-                shh += wa * (hA.x * hA.x + hA.y * hA.y) + we * (hE.x * hE.x + hE.y * hE.y);
-                rA = {wa * (a.x - hA.x), wa * (a.y - hA.y)};
-                rE = {we * (e.x - hE.x), we * (e.y - hE.y)};
-            }
-            // conjugate for the adjoint transform: c = conj(FFT(conj(r)))
-            bufA[idx] = {rA.x, -rA.y};
-            bufE[idx] = {rE.x, -rE.y};
-            if (useT) {
-                const C hT = cscale(bufT[idx], g.scale);
-                C rT = {0.0, 0.0};
-                if (kk >= 0 && kk < win.W) {
-                    const C t = dT[win.data_off + kk];
-                    const double wt = wT[win.data_off + kk];
-                    sdh += wt * (t.x * hT.x + t.y * hT.y);
-                    shh += wt * (hT.x * hT.x + hT.y * hT.y);
-                    rT = {wt * (t.x - hT.x), wt * (t.y - hT.y)};
-                }
-                bufT[idx] = {rT.x, -rT.y};
-            }
-        }
-        sdh = wsum(sdh) * (4.0 / T);
-        shh = wsum(shh) * (4.0 / T);
-        __syncwarp();
-        // (3) bit-reversal permutation in place, then the same forward FFT
-        for (int i = lane; i < N; i += 32) {
-            const int j = (int)(__brev((unsigned)i) >> (32 - g.logN));
-            if (i < j) {
-                const C ta = bufA[i];
-                bufA[i] = bufA[j];
-                bufA[j] = ta;
-                const C te = bufE[i];
-                bufE[i] = bufE[j];
-                bufE[j] = te;
-                if (useT) {
-                    const C tt = bufT[i];
-                    bufT[i] = bufT[j];
-                    bufT[j] = tt;
-                }
-            }
-        }
-        __syncwarp();
-        fft_inplace(N, g.logN, tw, bufA, bufE, bufT, lane);
-        // (4) reverse-mode sweep: the adjoint of sample n is c_n = conj(buf[n])
-        Acc acc = {0.0, 0.0, 0.0, 0.0, 0.0, {0.0, 0.0}, {0.0, 0.0}};
-        for (int n = lane; n < N; n += 32) {
-            const C cA = {bufA[n].x, -bufA[n].y}, cE = {bufE[n].x, -bufE[n].y};
-            const C cT = useT ? C{bufT[n].x, -bufT[n].y} : C{0.0, 0.0};
-            sample_adjoint(c, g, tab, n, cA, cE, cT, useT, acc);
-        }
-        double gacc[K];
-        gacc[0] = acc.f0;
-        gacc[1] = acc.fd;
-        gacc[2] = acc.beta;
-        gacc[3] = acc.lam;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) gacc[4 + k] = redot(acc.al, c.al_i[k]) + redot(acc.ga, c.ga_i[k]);
-        gacc[7] = acc.phi0;
-#pragma unroll
-        for (int k = 0; k < K; ++k) gacc[k] = wsum(gacc[k]) * (2.0 / (double)N);
-        if (lane == 0) {
-            if (logL_out) logL_out[cidx] = sdh - 0.5 * shh - 0.5 * dd;
-#pragma unroll
-            for (int k = 0; k < K; ++k) grad_out[8 * cidx + k] = gacc[k];
         }
         __syncwarp();
     }
@@ -555,12 +715,13 @@ int launch_grad_fp64(gb_ctx* ctx, const Plan& plan, const double* dA, const doub
                      const double* wE, const double* theta, double* logL, double* grad, const double* dT,
                      const double* wT, cudaStream_t s) {
     if (plan.n_tiles == 0) return GB_OK;
-    const size_t smem = sizeof(C) * kTwiddles + sizeof(double) * kWarpsG + sizeof(CandG) * kWarpsG * 32 +
+    const size_t smem = sizeof(FxTw) * kTwiddles + sizeof(double) * kWarpsG +
+                        (sizeof(CandGT) + sizeof(double) * kSumsG) * kWarpsG * kCapG +
                         sizeof(C) * kWarpsG * (dT ? 3 : 2) * (size_t)plan.n_max;
     cudaError_t e = cudaFuncSetAttribute(grad64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(ctx, e, "grad64: smem attribute");
     grad64_kernel<<<plan.n_tiles, kWarpsG * 32, smem, s>>>(plan.d_win, plan.d_tiles, tabset64(ctx),
-                                                           (const C*)ctx->d_tw64, ctx->obs.T_obs,
+                                                           (const C*)ctx->d_tw64, tabset_fx(ctx), ctx->obs.T_obs,
                                                            transfer_frequency(ctx), (const C*)dA, (const C*)dE,
                                                            wA, wE, theta, logL, grad, (const C*)dT, wT,
                                                            ctx->d_status, plan.n_max);

@@ -91,3 +91,44 @@ def test_mixed_forms_in_one_call(n):
     again = ctx.loglik_rows(wins, *args, dev(th), rows, lo, hi)
     for a, b in zip(again, got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("f0,fdot,N", [c for c in CASES if c[0] > 0 and c[2] <= 512])
+@pytest.mark.parametrize("aet", [False, True])
+def test_gradients_at_range_edges(f0, fdot, N, aet):
+    """Against the oracle's autodiff to the repository's 1e-9 of the gradient's norm (natural units)."""
+    T = 0.5 * wk.YEAR
+    n = 5
+    th = candidates(f0, fdot, n, N + 1)
+    th[1, 0] *= 1.01               # outside the window: zero gradient
+    qc = int(f0 * T + 0.5 * fdot * T * T)
+    W = N + 9
+    win = [(qc - W // 2, W, N, 0, 0, n)]
+    rng = np.random.default_rng(N)
+    d = [(rng.standard_normal(W) + 1j * rng.standard_normal(W)) * 1e-19 for _ in range(3)]
+    w = [rng.uniform(0.5, 1.5, W) * 1e41 for _ in range(3)]
+    dev = lambda x: torch.as_tensor(x, device="cuda")  # noqa: E731
+    ctx = api.Context(T)
+    if aet:
+        logL, g = ctx.loglik_grad_aet(win, *[dev(x) for x in d], *[dev(x) for x in w], dev(th))
+        ref_l, ref = gb.loglik_grad_aet(win, *d, *w, th, T)
+    else:
+        logL, g = ctx.loglik_grad(win, dev(d[0]), dev(d[1]), dev(w[0]), dev(w[1]), dev(th))
+        ref_l, ref = gb.loglik_grad(win, d[0], d[1], w[0], w[1], th, T)
+    scale = np.stack([np.full(n, 1 / T), np.full(n, 1 / T ** 2)] + [np.ones(n)] * 2 + [th[:, 4]] + [np.ones(n)] * 3, 1)
+    g, ref = g.cpu().numpy() * scale, np.asarray(ref) * scale
+    norm = np.linalg.norm(ref, axis=1)
+    assert np.all(np.linalg.norm(g - ref, axis=1) <= 1e-9 * np.maximum(norm, 1e-300) + (norm == 0) * 1e-300)
+    np.testing.assert_allclose(logL.cpu().numpy(), np.asarray(ref_l), rtol=1e-10)
+
+
+def test_gradient_of_non_finite_data_is_nan():
+    T, N, n = 0.5 * wk.YEAR, 64, 3
+    th = candidates(2e-3, 1e-17, n, 3)
+    win = [(int(2e-3 * T) - N // 2, N, N, 0, 0, n)]
+    d = torch.full((N,), 1e-19 + 0j, dtype=torch.complex128, device="cuda")
+    w = torch.full((N,), 1e41, dtype=torch.float64, device="cuda")
+    bad = d.clone()
+    bad[N // 2] = float("nan")
+    _, g = api.Context(T).loglik_grad(win, bad, d, w, w, torch.as_tensor(th, device="cuda"))
+    assert torch.isnan(g).all()
