@@ -162,22 +162,33 @@ class _Layout:
 
     def __init__(self, windows):
         self.n = len(windows)
-        try:   # integers, converted in bulk
-            if self.n == 0 or set(map(len, windows)) != {6}:
-                raise TypeError
-            t = np.array(array.array("q", itertools.chain.from_iterable(windows)), dtype=np.int64).reshape(self.n, 6)
-            rec = np.zeros(self.n, dtype=_WINDOW_DTYPE)
-            for k, name in enumerate(("k0", "W", "N", "data_off", "cand_off", "n_cand")):
-                rec[name] = t[:, k]
-            self.arr = (Window * self.n).from_buffer_copy(rec)
-        except (TypeError, OverflowError):
+        t = None
+        if self.n >= 64:   # bulk conversion; row by row costs less below
+            try:
+                if set(map(len, windows)) != {6}:
+                    raise TypeError
+                t = np.array(array.array("q", itertools.chain.from_iterable(windows)), dtype=np.int64)
+                t = t.reshape(self.n, 6)
+                rec = np.zeros(self.n, dtype=_WINDOW_DTYPE)
+                for k, name in enumerate(("k0", "W", "N", "data_off", "cand_off", "n_cand")):
+                    rec[name] = t[:, k]
+                self.arr = (Window * self.n).from_buffer_copy(rec)
+            except (TypeError, OverflowError):
+                t = None
+        if t is None:
             rows = [tuple(int(x) for x in w) for w in windows]
             self.arr = windows_array(rows)
-            t = np.array(rows, dtype=np.int64).reshape(self.n, 6)
-        off, cnt = t[:, 4], t[:, 5]
-        gapless = bool((cnt >= 0).all()) and np.array_equal(off, np.cumsum(cnt) - cnt)
-        self.covered = int(cnt.sum()) if gapless else -1
-        self.kmax = int(max(1, cnt.max(initial=1)))
+            at = 0
+            for w in rows:
+                if at >= 0:
+                    at = at + w[5] if w[4] == at and w[5] >= 0 else -1
+            self.covered = at
+            self.kmax = max([1] + [w[5] for w in rows])
+        else:
+            off, cnt = t[:, 4], t[:, 5]
+            gapless = bool((cnt >= 0).all()) and np.array_equal(off, np.cumsum(cnt) - cnt)
+            self.covered = int(cnt.sum()) if gapless else -1
+            self.kmax = int(max(1, cnt.max()))
 
 
 class Context:

@@ -3,6 +3,7 @@ scaling of Eq. 8, the Alg. 1 segments and the full-band window layout."""
 import math
 
 import numpy as np
+import pytest
 
 from paper_2307_03763_gb300 import workloads as wk
 
@@ -83,6 +84,19 @@ def test_n_for_band_is_the_smallest_power_of_two():
         n = wk.n_for_band(f, T)
         bins = 2 * float(wk.bandwidth_max(f, T, 1.0)) * T
         assert n & (n - 1) == 0 and n >= 32 and n >= bins and (n == 32 or n / 2 < bins)
+
+
+@pytest.mark.parametrize("n", [63, 64, 65])
+def test_layout_conversion_in_bulk_and_by_row(n):
+    from paper_2307_03763_gb300 import api
+    rows = [(10 ** 10 + i, 33, 64, 33 * i, 2 * i, 2) for i in range(n)]
+    lay = api._Layout(rows)
+    assert bytes(lay.arr) == bytes(api.windows_array(rows)) and (lay.covered, lay.kmax) == (2 * n, 2)
+    rows[n // 2] = rows[n // 2][:5] + (3,)
+    assert (api._Layout(rows).covered, api._Layout(rows).kmax) == (-1, 3)
+    assert bytes(api._Layout([tuple(float(x) for x in r) for r in rows]).arr) == bytes(api.windows_array(rows))
+    with pytest.raises(ValueError):
+        api._Layout(rows[:-1] + [(1, 2, 3)])
 
 
 def test_layouts_are_kept_by_value():
