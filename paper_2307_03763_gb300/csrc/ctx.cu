@@ -259,8 +259,8 @@ static cudaError_t alloc_mixed_scratch(Plan& p, const gb_window_t* win, int n_wi
     if (e == cudaSuccess) e = cudaMemcpy(p.d_meta, meta.data(), sizeof(WinMeta) * meta.size(), cudaMemcpyHostToDevice);
     // float window copies: A and E, then T (filled only when the T channel is given)
     if (e == cudaSuccess) e = cudaMalloc(&p.d_prep, 2 * sizeof(Win32) * (size_t)(off > 0 ? off : 1));
-    if (e == cudaSuccess) e = cudaMalloc(&p.d_head, 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(p.d_head, 0, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&p.d_head, kParts * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(p.d_head, 0, kParts * sizeof(int));
     return e;
 }
 
@@ -307,12 +307,15 @@ int get_plan(gb_ctx* ctx, int prec, const gb_window_t* win, int32_t n_win, int t
         const gb_window_t& g = win[w];
         n_max = std::max(n_max, g.N);
         w_max = std::max(w_max, g.W);
-        for (int64_t c = 0; c < g.n_cand; c += tile_cands) {
+        // the mixed gradient's items hold at most 16 candidates for N >= 512,
+        // which leaves room for two CTAs per SM in place of one
+        const int most = prec == GB_MIXED + 16 && g.N >= 512 ? std::min(tile_cands, 16) : tile_cands;
+        for (int64_t c = 0; c < g.n_cand; c += most) {
             Tile t;
             t.win = w;
             t.pad = 0;
             t.c_begin = g.cand_off + c;
-            t.c_end = g.cand_off + std::min<int64_t>(g.n_cand, c + tile_cands);
+            t.c_end = g.cand_off + std::min<int64_t>(g.n_cand, c + most);
             tiles.push_back(t);
             cost.push_back((double)(t.c_end - t.c_begin) * g.N * (log2_size(g.N) + 12));
         }
@@ -320,39 +323,38 @@ int get_plan(gb_ctx* ctx, int prec, const gb_window_t* win, int32_t n_win, int t
     std::vector<int> order(tiles.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-    // mixed plans: items of windows with N >= 512 first (their own kernel)
-    int n_large = 0;
-    if ((prec & 15) == GB_MIXED) {
-        std::stable_partition(order.begin(), order.end(), [&](int a) { return win[tiles[a].win].N >= 512; });
-        for (const Tile& t : tiles) n_large += win[t.win].N >= 512 ? 1 : 0;
-    }
     std::vector<Tile> sorted(tiles.size());
     for (size_t i = 0; i < order.size(); ++i) sorted[i] = tiles[order[i]];
-    if ((prec == GB_MIXED || prec == GB_MIXED + 16) && tile_cands >= 4) {
-        // The persistent warps take the items in this order, so the last ones
-        // set the tail.  With R warps resident (likelihood: 16 per SM for
-        // N <= 256, 8 for N >= 512; gradient: 8 and 4), the last R/2 items of
-        // each range are split into halves
-        // and the last R/4 of those halves into halves again: the last round
-        // is shared out in smaller items, while the extra per-item set-ups
-        // stay few (a list-scheduling model of the queue with the measured
-        // set-up cost puts this near the best split; splitting the last 2R
-        // items costs more in set-ups than it saves).
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms <= 0)
-            sms = 152;
-        std::vector<Tile> large(sorted.begin(), sorted.begin() + n_large), small(sorted.begin() + n_large, sorted.end());
-        const size_t per_sm = prec == GB_MIXED ? 16 : 8;
-        const size_t r_large = (size_t)sms * per_sm / 2, r_small = (size_t)sms * per_sm;
-        split_last(large, r_large / 2);
-        split_last(large, r_large / 4);
-        split_last(small, r_small / 2);
-        split_last(small, r_small / 4);
-        n_large = (int)large.size();
-        sorted = large;
-        sorted.insert(sorted.end(), small.begin(), small.end());
+    int n_part[kParts] = {}, cap_part[kParts] = {};
+    if ((prec & 15) == GB_MIXED) {
+        std::vector<Tile> part[kParts];
+        for (const Tile& t : sorted) part[part_of(win[t.win].N)].push_back(t);
+        if (tile_cands >= 4) {
+            // The persistent warps take the items in this order, so the last
+            // ones set the tail.  With R warps resident, the last R/2 items of
+            // each part are split into halves and the last R/4 of those halves
+            // into halves again: the last round is shared out in smaller
+            // items, while the extra per-item set-ups stay few (a
+            // list-scheduling model of the queue with the measured set-up cost
+            // puts this near the best split; splitting the last 2R items costs
+            // more in set-ups than it saves).
+            int sms = 0;
+            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms <= 0)
+                sms = 152;
+            const int warps_sm[2][kParts] = {{8, 8, 16}, {8, 8, 8}};   // likelihood, gradient
+            for (int p = 0; p < kParts; ++p) {
+                const size_t R = (size_t)sms * warps_sm[prec == GB_MIXED ? 0 : 1][p];
+                split_last(part[p], R / 2);
+                split_last(part[p], R / 4);
+            }
+        }
+        sorted.clear();
+        for (int p = 0; p < kParts; ++p) {
+            n_part[p] = (int)part[p].size();
+            for (const Tile& t : part[p]) cap_part[p] = std::max(cap_part[p], (int)(t.c_end - t.c_begin));
+            sorted.insert(sorted.end(), part[p].begin(), part[p].end());
+        }
     }
-
     if (prec == GB_FP64 && tile_cands >= 32) {
         // CTAs take their tiles in this order too (three resident per SM): the
         // last half-round in halves, half of those in halves again (with tiles
@@ -378,7 +380,8 @@ int get_plan(gb_ctx* ctx, int prec, const gb_window_t* win, int32_t n_win, int t
     p.n_tiles = (int)sorted.size();
     p.n_max = n_max;
     p.w_max = w_max;
-    p.n_large = n_large;
+    std::copy(n_part, n_part + kParts, p.n_part);
+    std::copy(cap_part, cap_part + kParts, p.cap_part);
     p.tile_cands = tile_cands;
     p.win.assign(win, win + n_win);
     p.last_use = ctx->clock;

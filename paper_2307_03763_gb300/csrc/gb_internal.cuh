@@ -118,6 +118,16 @@ struct Win32 {
     float2 w;     // (wA, wE)
 };
 
+// The mixed kernels run in three parts by template length, N = 1,024, N = 512
+// and N <= 256, each with its own work queue and the shared memory that its
+// buffers need.  N = 512 in one part with N = 1,024, and so with twice the
+// buffers and half the L1: 512 windows over the band 15.68 ms against 15.26,
+// the gradient of 2,048 windows of 16 rows 1.07 ms against 0.88.  An
+// instantiation of its own for N = 512, three CTAs per SM: 15.72 ms.
+constexpr int kParts = 3;
+inline int part_of(int N) { return N >= 1024 ? 0 : N >= 512 ? 1 : 2; }
+inline int part_nmax(int part, int n_max) { return part == 0 ? 1024 : part == 1 ? 512 : n_max < 256 ? n_max : 256; }
+
 struct Plan {
     uint64_t key = 0;
     int prec = -1;
@@ -126,7 +136,8 @@ struct Plan {
     int n_max = 0;
     int w_max = 0;
     long long n_prep = 0;           // total window bins (scratch entries)
-    int n_large = 0;                // mixed plans: items with N >= 512 come first
+    int n_part[kParts] = {};        // mixed plans: items of each kernel part, in this order
+    int cap_part[kParts] = {};      // and the candidates of its largest item
     int tile_cands = 0;             // candidates per work item at most
     std::vector<gb_window_t> win;   // host copy of the layout: a lookup compares it, not only the hash
     gb_window_t* d_win = nullptr;
@@ -134,7 +145,7 @@ struct Plan {
     // scratch of the mixed-precision path (owned by the plan)
     WinMeta* d_meta = nullptr;
     Win32* d_prep = nullptr;
-    int* d_head = nullptr;          // work-queue head
+    int* d_head = nullptr;          // work-queue heads, one per part
     uint64_t last_use = 0;
 };
 
@@ -293,8 +304,8 @@ int launch_loglik_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const d
                         const double* wA, const double* wE, const double* theta, double* logL,
                         double* dh, double* hh, double* dh_im, const double* dT, const double* wT,
                         cudaStream_t s);
-// the persistent likelihood kernel with the phase output and/or the T channel
-// (part 0: N >= 512, part 1: N <= 256), compiled in mixed_variants.cu
+// the persistent likelihood kernel of a part (part_of) with the phase output
+// and/or the T channel, compiled in mixed_variants.cu
 const void* mixed_kernel_fn_variant(int part, bool im, bool t3);
 const void* mixed_kernel_fn_t(int part, bool im);            // mixed_variants_t.cu
 const void* grad_mixed_kernel_fn_t(int part);                // mixed_grad_t.cu, the gradient with T

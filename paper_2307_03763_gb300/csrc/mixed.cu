@@ -67,11 +67,11 @@ __global__ void __launch_bounds__(kWarpsMx * 32) waveform_mixed_kernel(
     }
 }
 
-// Part 0 drains the N >= 512 queue, part 1 the N <= 256 queue; the variants
-// with the phase output or the T channel are compiled in mixed_variants.cu.
+// The kernel that drains a part's queue; the variants with the phase output or
+// the T channel are compiled in mixed_variants.cu.
 const void* mixed_kernel_fn(int part, bool im, bool t3) {
     if (im || t3) return mixed_kernel_fn_variant(part, im, t3);
-    return part == 0 ? (const void*)loglik_mixed_kernel<32, false, false> : (const void*)loglik_mixed_kernel<8, false, false>;
+    return part < 2 ? (const void*)loglik_mixed_kernel<32, false, false> : (const void*)loglik_mixed_kernel<8, false, false>;
 }
 
 }  // namespace
@@ -97,16 +97,14 @@ int launch_loglik_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const d
         e = cudaEventRecord(ev_start, s);
         if (e != cudaSuccess) return cuda_error(ctx, e, "loglik_mixed: kernel start event");
     }
-    // two persistent launches drain the two queues: N >= 512 items, then N <= 256
-    const int n_small = plan.n_tiles - plan.n_large;
-    for (int part = 0; part < 2; ++part) {
-        const int n_items = part == 0 ? plan.n_large : n_small;
+    // one persistent launch per part drains its queue, the longest templates first
+    int first = 0, chain = 0;
+    size_t held = 0;
+    for (int part = 0; part < kParts; first += plan.n_part[part], ++part) {
+        const int n_items = plan.n_part[part];
         if (n_items == 0) continue;
-        const int nmax = part == 0 ? 1024 : (plan.n_max < 256 ? plan.n_max : 256);
-        const size_t epi_bytes = dh_im ? sizeof(Epi<true>) : sizeof(Epi<false>);
-        const size_t cap = t3 ? kCapT : 32;
-        const size_t smem = (sizeof(CandMix) + epi_bytes) * kWarpsMx * cap + sizeof(float2) * kWarpsMx * 2 * (size_t)nmax +
-                            (t3 ? sizeof(float2) * kWarpsMx * (size_t)nmax : 0);
+        const int nmax = part_nmax(part, plan.n_max);
+        const size_t smem = kWarpsMx * warp_smem(t3 ? 3 : 2, nmax, sizeof(CandMix), plan.cap_part[part]);
         const void* kfn = mixed_kernel_fn(part, dh_im != nullptr, t3);
         e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(ctx, e, "loglik_mixed: smem attribute");
@@ -115,11 +113,13 @@ int launch_loglik_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const d
         int grid = sms * bpsm;
         const int need = (n_items + kWarpsMx - 1) / kWarpsMx;
         if (grid > need) grid = need;
-        const Tile* items = plan.d_tiles + (part == 0 ? 0 : plan.n_large);
-        int* head = plan.d_head + (part == 0 ? 1 : 0);
-        e = launch_mixed_part(kfn, grid, smem, s, plan.d_win, plan.d_meta, plan.d_prep, items, n_items, head,
-                              tabset32(ctx), (const float2*)ctx->d_tw32, ctx->obs.T_obs, transfer_frequency(ctx),
-                              theta, logL, dh, hh, dh_im, ctx->d_status, nmax, ctx->budget_ns, plan.n_prep);
+        const bool dependent = chain == 0 ? !ev_start : held <= kHeldMax;
+        e = launch_mixed_part(kfn, grid, smem, s, plan.d_win, plan.d_meta, plan.d_prep, plan.d_tiles + first, n_items,
+                              plan.d_head + part, tabset32(ctx), (const float2*)ctx->d_tw32, ctx->obs.T_obs,
+                              transfer_frequency(ctx), theta, logL, dh, hh, dh_im, ctx->d_status, nmax,
+                              ctx->budget_ns, plan.n_prep, chain, dependent);
+        held = smem * bpsm;
+        ++chain;
         ++ctx->launches;
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_error(ctx, e, "loglik_mixed launch");
@@ -184,7 +184,7 @@ constexpr size_t kNaOffItems = na_round(kNaOffWin + sizeof(gb_window_t) * kNaMax
 constexpr size_t kNaOffMeta = na_round(kNaOffItems + sizeof(Tile) * kNaMaxItems);
 constexpr size_t kNaOffPrep = na_round(kNaOffMeta + sizeof(WinMeta) * kNaMaxWindows);
 constexpr size_t kNaOffHead = na_round(kNaOffPrep + sizeof(Win32) * kNaMaxBins);
-constexpr size_t kNaBytes = na_round(kNaOffHead + 4 * sizeof(int));   // two queue heads, status
+constexpr size_t kNaBytes = na_round(kNaOffHead + (kParts + 1) * sizeof(int));   // queue heads, status
 
 // 8.7 MB per device, kept until the process exits
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
@@ -330,11 +330,11 @@ extern "C" int gb_loglik_mixed_noalloc(const gb_obs_t* obs, const gb_window_t* w
         d.T = obs->T_obs;
         d.L = obs->arm_L;
     }
-    // work items (windows with N >= 512 first) and window offsets, staged on the host
-    int n_large = 0, k = 0;
-    for (int pass = 0; pass < 2; ++pass)
+    // work items (part by part) and window offsets, staged on the host
+    int n_part[kParts] = {}, k = 0;
+    for (int part = 0; part < kParts; ++part)
         for (int i = 0; i < n_win; ++i) {
-            if ((win[i].N >= 512) != (pass == 0)) continue;
+            if (part_of(win[i].N) != part) continue;
             for (int64_t c = 0; c < win[i].n_cand; c += per) {
                 Tile t;
                 t.win = i;
@@ -342,7 +342,7 @@ extern "C" int gb_loglik_mixed_noalloc(const gb_obs_t* obs, const gb_window_t* w
                 t.c_begin = win[i].cand_off + c;
                 t.c_end = win[i].cand_off + std::min<int64_t>(win[i].n_cand, c + per);
                 g_na_items[k++] = t;
-                if (pass == 0) ++n_large;
+                ++n_part[part];
             }
         }
     long long off = 0;
@@ -359,7 +359,7 @@ extern "C" int gb_loglik_mixed_noalloc(const gb_obs_t* obs, const gb_window_t* w
     WinMeta* d_meta = (WinMeta*)(b + kNaOffMeta);
     Win32* d_prep = (Win32*)(b + kNaOffPrep);
     int* d_head = (int*)(b + kNaOffHead);
-    int* d_status = d_head + 2;
+    int* d_status = d_head + kParts;
     e = cudaMemcpyAsync(d_win, win, sizeof(gb_window_t) * (size_t)n_win, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_items, g_na_items, sizeof(Tile) * (size_t)k, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
@@ -371,22 +371,22 @@ extern "C" int gb_loglik_mixed_noalloc(const gb_obs_t* obs, const gb_window_t* w
     prep_mixed_kernel<<<n_win, 256, 0, s>>>(d_win, d_meta, d_prep, (const double2*)dA, (const double2*)dE, wA, wE,
                                             nullptr, nullptr, 0LL, obs->T_obs, fstar, d_head);
     e = cudaGetLastError();
-    for (int part = 0; part < 2 && e == cudaSuccess; ++part) {
-        const int n_items = part == 0 ? n_large : k - n_large;
+    int first = 0, chain = 0;
+    for (int part = 0; part < kParts && e == cudaSuccess; first += n_part[part], ++part) {
+        const int n_items = n_part[part];
         if (n_items == 0) continue;
-        const int nmax = part == 0 ? 1024 : (n_max < 256 ? n_max : 256);
-        const size_t smem =
-            (sizeof(CandMix) + sizeof(Epi<false>)) * kWarpsMx * 32 + sizeof(float2) * kWarpsMx * 2 * (size_t)nmax;
+        const int nmax = part_nmax(part, n_max);
+        const size_t smem = kWarpsMx * warp_smem(2, nmax, sizeof(CandMix), per);
         const void* kfn = mixed_kernel_fn(part, false, false);
         e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) break;
         int grid = sms * resident_blocks(kfn, kWarpsMx * 32, smem);
         const int need = (n_items + kWarpsMx - 1) / kWarpsMx;
         if (grid > need) grid = need;
-        const Tile* it = d_items + (part == 0 ? 0 : n_large);
-        int* head = d_head + (part == 0 ? 1 : 0);
-        e = launch_mixed_part(kfn, grid, smem, s, d_win, d_meta, d_prep, it, n_items, head, tabs, (const float2*)tw32,
-                              obs->T_obs, fstar, theta, logL, dh, hh, nullptr, d_status, nmax, 0ULL, 0LL);
+        e = launch_mixed_part(kfn, grid, smem, s, d_win, d_meta, d_prep, d_items + first, n_items, d_head + part, tabs,
+                              (const float2*)tw32, obs->T_obs, fstar, theta, logL, dh, hh, nullptr, d_status, nmax, 0ULL,
+                              0LL, chain, true);
+        ++chain;
         if (e == cudaSuccess) e = cudaGetLastError();
     }
     if (e == cudaSuccess && status) e = cudaMemcpyAsync(status, d_status, sizeof(int32_t), cudaMemcpyDeviceToDevice, s);

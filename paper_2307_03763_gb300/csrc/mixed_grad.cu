@@ -17,33 +17,37 @@ int launch_grad_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const dou
     if (e != cudaSuccess) return cuda_error(ctx, e, "prep_mixed launch");
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    const int n_small = plan.n_tiles - plan.n_large;
-    for (int part = 0; part < 2; ++part) {
-        const int n_items = part == 0 ? plan.n_large : n_small;
+    int first = 0, chain = 0;
+    size_t held = 0;
+    for (int part = 0; part < kParts; first += plan.n_part[part], ++part) {
+        const int n_items = plan.n_part[part];
         if (n_items == 0) continue;
-        const int nmax = part == 0 ? 1024 : (plan.n_max < 256 ? plan.n_max : 256);
-        const size_t smem = (sizeof(CandGx) + sizeof(EpiG)) * kWarpsMx * 32 +
-                            sizeof(float2) * kWarpsMx * (t3 ? 3 : 2) * (size_t)nmax;
+        const int nmax = part_nmax(part, plan.n_max);
+        const size_t smem = kWarpsMx * warp_smem(t3 ? 3 : 2, nmax, sizeof(CandGx), plan.cap_part[part]);
         const void* kfn = t3 ? grad_mixed_kernel_fn_t(part)
-                             : (part == 0 ? (const void*)grad_mixed_kernel<32, false>
-                                          : (const void*)grad_mixed_kernel<8, false>);
+                             : part < 2 ? (const void*)grad_mixed_kernel<32, false>
+                                        : (const void*)grad_mixed_kernel<8, false>;
         e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(ctx, e, "grad_mixed: smem attribute");
-        int grid = sms * resident_blocks(kfn, kWarpsMx * 32, smem);
+        const int bpsm = resident_blocks(kfn, kWarpsMx * 32, smem);
+        int grid = sms * bpsm;
         const int need = (n_items + kWarpsMx - 1) / kWarpsMx;
         if (grid > need) grid = need;
-        const Tile* items = plan.d_tiles + (part == 0 ? 0 : plan.n_large);
-        int* head = plan.d_head + (part == 0 ? 1 : 0);
+        const Tile* items = plan.d_tiles + first;
+        int* head = plan.d_head + part;
         TabSet32 tabs = tabset32(ctx);
         const float2* tw = (const float2*)ctx->d_tw32;
         double Tobs = ctx->obs.T_obs, fstar = transfer_frequency(ctx);
         int* status = ctx->d_status;
         unsigned long long budget = ctx->budget_ns;
         long long n_prep = plan.n_prep;
-        int n_it = n_items, n_mx = nmax;
+        int n_it = n_items, n_mx = nmax, warp_bytes = (int)(smem / kWarpsMx);
         void* args[] = {(void*)&plan.d_win, (void*)&plan.d_meta, (void*)&plan.d_prep, (void*)&items, &n_it, &head,
-                        &tabs, &tw, &Tobs, &fstar, (void*)&theta, &logL, &grad, &status, &n_mx, &budget, &n_prep};
-        e = cudaLaunchKernel(kfn, dim3(grid), dim3(kWarpsMx * 32), args, smem, s);
+                        &tabs, &tw, &Tobs, &fstar, (void*)&theta, &logL, &grad, &status, &n_mx, &budget, &n_prep,
+                        &chain, &warp_bytes};
+        e = launch_chained(kfn, grid, smem, s, args, chain == 0 || held <= kHeldMax);
+        held = smem * bpsm;
+        ++chain;
         ++ctx->launches;
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_error(ctx, e, "grad_mixed launch");

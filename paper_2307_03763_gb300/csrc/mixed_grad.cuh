@@ -424,6 +424,8 @@ struct EpiG {
     float vp[2][2], vq[2][2];   // [re, im][hi, lo]
 };
 
+static_assert(sizeof(EpiG) <= offsetof(CandMix, f0), "the sums leave the candidate's A and bad in place");
+
 // Forward FFT of one channel, window inner products, residual (conjugated) in
 // natural bin order in buf, then the adjoint FFT leaving c^_n = buf[n].
 template <int R>
@@ -596,54 +598,60 @@ __device__ void residual_adjoint_nat(float4* buf, const OrbitTables32& tab, cons
     __syncwarp();
 }
 
-// resident CTAs per SM the N <= 256 instantiation is compiled for (register cap)
+// resident CTAs per SM the kernel is compiled for (register cap)
 #ifndef GB_GRAD_MINB
 #define GB_GRAD_MINB 2
 #endif
-
 template <int RMAX, bool T3>
-__global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_GRAD_MINB : 1) grad_mixed_kernel(
+__global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel(
     const gb_window_t* __restrict__ wins, const WinMeta* __restrict__ meta, const Win32* __restrict__ prep,
     const Tile* __restrict__ items, int n_items, int* head, TabSet32 tabs, const float2* __restrict__ tw1024,
     double T, double fstar, const double* __restrict__ theta, double* __restrict__ logL,
-    double* __restrict__ grad, int* status, int n_max, unsigned long long budget_ns, long long n_prep) {
+    double* __restrict__ grad, int* status, int n_max, unsigned long long budget_ns, long long n_prep,
+    int chain, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    CandGx* cands = (CandGx*)smem_raw + warp * 32;
-    EpiG* epi = (EpiG*)((CandGx*)smem_raw + kWarpsMx * 32) + warp * 32;
-    float2* bufA = (float2*)((EpiG*)((CandGx*)smem_raw + kWarpsMx * 32) + kWarpsMx * 32) + (size_t)warp * 2 * n_max;
+    // per warp: the channels' buffers and the candidates of the item
+    float2* bufA = (float2*)(smem_raw + (size_t)warp * warp_bytes);
     float2* bufE = bufA + n_max;
-    // T3: one more buffer per warp, for T
-    float2* bufT = T3 ? (float2*)((EpiG*)((CandGx*)smem_raw + kWarpsMx * 32) + kWarpsMx * 32) +
-                            (size_t)kWarpsMx * 2 * n_max + (size_t)warp * n_max
-                      : nullptr;
+    float2* bufT = T3 ? bufE + n_max : nullptr;
+    CandGx* cands = (CandGx*)(bufA + (T3 ? 3 : 2) * n_max);
     const LaneTw ltw = lane_twiddles(lane);
     const float Tf = (float)T, inv_fstar = (float)(1.0 / fstar);
-    const unsigned long long t0 = global_ns();
+    const unsigned long long t0 = budget_ns != 0ULL ? global_ns() : 0ULL;
+    // first items and waits as in loglik_mixed_kernel
+    const int fixed = chain == 0 ? (int)gridDim.x * kWarpsMx : 0;
+    bool waited = chain != 0;
+    if (waited) pdl_launch_dependents();
     for (;;) {
         // a warp past the time budget takes no further item and flags it
-        int item = 0;
+        int item = blockIdx.x * kWarpsMx + warp;
         if (lane == 0) {
             if (budget_ns != 0ULL && global_ns() - t0 > budget_ns) {
                 atomicOr(status, kStatusBudget);
                 item = n_items;
-            } else {
-                item = atomicAdd(head, 1);
+            } else if (waited) {
+                item = fixed + atomicAdd(head, 1);
             }
         }
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= n_items) break;
         const Tile t = items[item];
         const gb_window_t win = wins[t.win];
-        const WinMeta wm = meta[t.win];
-        const Win32* pw = prep + wm.prep_off;
         const int N = win.N;
         const OrbitTables32 tab = tabs.t[__ffs(N) - 6];
         const int cnt = (int)(t.c_end - t.c_begin);
-        const bool useT = T3 && wm.use_t;
-        const Win32* pwT = prep + n_prep + wm.prep_off;
         if (lane < cnt) setup_grad_mixed(theta + 8 * (t.c_begin + lane), T, fstar, cands[lane]);
         __syncwarp();
+        if (!waited) {
+            pdl_wait();
+            pdl_launch_dependents();
+            waited = true;
+        }
+        const WinMeta wm = after_wait(meta)[t.win];
+        const Win32* pw = after_wait(prep) + wm.prep_off;
+        const bool useT = T3 && wm.use_t;
+        const Win32* pwT = pw + n_prep;
         for (int i = 0; i < cnt; ++i) {
             const CandGx& g = cands[i];
             float sdh = 0.0f, cdh = 0.0f, shh = 0.0f, chh = 0.0f;
@@ -739,7 +747,8 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_GRAD_MINB : 1) g
                 warp_sum2(vp[q][0], vp[q][1], s.vp[q][0], s.vp[q][1]);
                 warp_sum2(vq[q][0], vq[q][1], s.vq[q][0], s.vq[q][1]);
             }
-            if (lane == 0) epi[i] = s;
+            __syncwarp();
+            if (lane == 0) *(EpiG*)&cands[i].m = s;   // over constants that are no longer needed
         }
         __syncwarp();
         if (lane < cnt) {
@@ -750,7 +759,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_GRAD_MINB : 1) g
                 for (int k = 0; k < 8; ++k) grad[8 * cidx + k] = nan("");
                 atomicOr(status, kStatusNonFinite);
             } else {
-                const EpiG& s = epi[lane];
+                const EpiG& s = *(const EpiG*)&g.m;
                 const double A = g.m.A, sig = wm.sig;
                 const double dh = A * (2.0 * sig / (double)N) * ((double)s.dh[0] + (double)s.dh[1]);
                 const double hh = A * A * (T * sig * sig / ((double)N * (double)N)) * ((double)s.hh[0] + (double)s.hh[1]);
@@ -772,6 +781,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_GRAD_MINB : 1) g
         }
         __syncwarp();
     }
+    pdl_wait();
 }
 
 }  // namespace

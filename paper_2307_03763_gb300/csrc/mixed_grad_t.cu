@@ -5,7 +5,7 @@
 namespace gb {
 
 const void* grad_mixed_kernel_fn_t(int part) {
-    return part == 0 ? (const void*)grad_mixed_kernel<32, true> : (const void*)grad_mixed_kernel<8, true>;
+    return part < 2 ? (const void*)grad_mixed_kernel<32, true> : (const void*)grad_mixed_kernel<8, true>;
 }
 
 }  // namespace gb

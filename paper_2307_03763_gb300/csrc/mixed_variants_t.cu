@@ -5,8 +5,8 @@
 namespace gb {
 
 const void* mixed_kernel_fn_t(int part, bool im) {
-    if (im) return part == 0 ? (const void*)loglik_mixed_kernel<32, true, true> : (const void*)loglik_mixed_kernel<8, true, true>;
-    return part == 0 ? (const void*)loglik_mixed_kernel<32, false, true> : (const void*)loglik_mixed_kernel<8, false, true>;
+    if (im) return part < 2 ? (const void*)loglik_mixed_kernel<32, true, true> : (const void*)loglik_mixed_kernel<8, true, true>;
+    return part < 2 ? (const void*)loglik_mixed_kernel<32, false, true> : (const void*)loglik_mixed_kernel<8, false, true>;
 }
 
 }  // namespace gb
