@@ -122,8 +122,7 @@ struct Win32 {
 // and N <= 256, each with its own work queue and the shared memory that its
 // buffers need.  N = 512 in one part with N = 1,024, and so with twice the
 // buffers and half the L1: 512 windows over the band 15.68 ms against 15.26,
-// the gradient of 2,048 windows of 16 rows 1.07 ms against 0.88.  An
-// instantiation of its own for N = 512, three CTAs per SM: 15.72 ms.
+// the gradient of 2,048 windows of 16 rows 1.07 ms against 0.88.
 constexpr int kParts = 3;
 inline int part_of(int N) { return N >= 1024 ? 0 : N >= 512 ? 1 : 2; }
 inline int part_nmax(int part, int n_max) { return part == 0 ? 1024 : part == 1 ? 512 : n_max < 256 ? n_max : 256; }

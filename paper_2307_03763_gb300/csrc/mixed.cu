@@ -71,7 +71,9 @@ __global__ void __launch_bounds__(kWarpsMx * 32) waveform_mixed_kernel(
 // the T channel are compiled in mixed_variants.cu.
 const void* mixed_kernel_fn(int part, bool im, bool t3) {
     if (im || t3) return mixed_kernel_fn_variant(part, im, t3);
-    return part < 2 ? (const void*)loglik_mixed_kernel<32, false, false> : (const void*)loglik_mixed_kernel<8, false, false>;
+    return part == 0   ? (const void*)loglik_mixed_kernel<32, false, false>
+           : part == 1 ? (const void*)loglik_mixed_kernel<16, false, false>
+                       : (const void*)loglik_mixed_kernel<8, false, false>;
 }
 
 }  // namespace

@@ -1466,11 +1466,6 @@ __global__ void prep_mixed_kernel(const gb_window_t* __restrict__ wins, WinMeta*
     }
 }
 
-// resident CTAs per SM the instantiations are compiled for (register caps)
-#ifndef GB_MIXED_MINB
-#define GB_MIXED_MINB 4
-#endif
-// RMAX: largest R = N/32 this instantiation handles (8: N <= 256; 32: N = 512, 1024)
 // the two channels' compensated sums added into one (true sums s - c)
 __device__ __forceinline__ void kahan_join(float& s, float& c, float s2, float c2) {
     float hi, e;
@@ -1479,8 +1474,21 @@ __device__ __forceinline__ void kahan_join(float& s, float& c, float s2, float c
     c = (c + c2) - e;
 }
 
+// RMAX: largest R = N/32 this instantiation handles (8: N <= 256; 16: N = 512;
+// 32: N = 512 and 1,024).  Bound by the FP32 pipe (65-70 % busy) and the
+// latencies that the resident warps leave open, so the register caps trade
+// registers for warps.  512 windows over the band, 4,100 candidates each:
+// 15.26 ms with 4 CTAs per SM for N <= 256 and the shared kernel for N = 512;
+// 14.97 ms with 5, 15.04 with 6; a kernel of its own for N = 512 takes off
+// 0.16 ms with 3 CTAs, 0.08 with 4, and adds 0.14 with 2.  With the T channel
+// neither pays (5.36 ms: 5.38 and 5.44).
+#ifndef GB_MIXED_MINB
+#define GB_MIXED_MINB 5
+#endif
 template <int RMAX, bool IM, bool T3>
-__global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_MIXED_MINB : 2) loglik_mixed_kernel(
+__global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIXED_MINB)
+                                                        : RMAX == 16 ? 3
+                                                                     : 2) loglik_mixed_kernel(
     const gb_window_t* __restrict__ wins, const WinMeta* __restrict__ meta, const Win32* __restrict__ prep,
     const Tile* __restrict__ items, int n_items, int* head, TabSet32 tabs, const float2* __restrict__ tw1024,
     double T, double fstar, const double* __restrict__ theta, double* __restrict__ logL,
@@ -1554,7 +1562,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8 ? GB_MIXED_MINB : 2) 
                             default: GB_FFT_INNER(8); break;
                         }
                     } else {
-                        if (N == 512)
+                        if (RMAX == 16 || N == 512)
                             GB_FFT_INNER(16);
                         else
                             GB_FFT_INNER(32);

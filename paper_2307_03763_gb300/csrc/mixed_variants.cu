@@ -8,7 +8,9 @@ namespace gb {
 
 const void* mixed_kernel_fn_variant(int part, bool im, bool t3) {
     if (t3) return mixed_kernel_fn_t(part, im);
-    return part < 2 ? (const void*)loglik_mixed_kernel<32, true, false> : (const void*)loglik_mixed_kernel<8, true, false>;
+    return part == 0   ? (const void*)loglik_mixed_kernel<32, true, false>
+           : part == 1 ? (const void*)loglik_mixed_kernel<16, true, false>
+                       : (const void*)loglik_mixed_kernel<8, true, false>;
 }
 
 }  // namespace gb
