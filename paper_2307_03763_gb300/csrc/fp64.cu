@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kWarps64 * 32, kMinCtas64) loglik64_kernel(
         for (int slot = lo + (int)blockIdx.y; slot < hi; slot += (int)gridDim.y) {
             const int64_t row = rows[win.cand_off + slot];
             if (row < win.cand_off || row >= win.cand_off + win.n_cand) continue;   // not this window's row
-            if (warp == 0) setup_warp(theta + 8 * row, g, cands[0], lane);
+            if (warp == 0) setup_warp(theta + 8 * row, 1, g, cands, lane);
             __syncthreads();
             if (cands[0].bad) {
                 if (threadIdx.x == 0) bad64(row, logL, dh_out, hh_out, dhi_out, status);
@@ -264,120 +264,192 @@ __global__ void __launch_bounds__(kWarps64 * 32, kMinCtas64) waveform64_kernel(
     }
 }
 
-// Window inner product <x|y> = (4/T) Re sum_k w_k x_k y_k* of two templates
-// (or data, y) over the window's bins, block-wide in a fixed order.  A
-// template is given by its buffers of bin values (natural order, at sw(index))
-// and carrier bin; bins it does not reach count zero.  `red` holds kWarps64
-// doubles.
-struct WinTpl {
-    const C64* A;
-    const C64* E;
-    long long q;
-};
-__device__ __forceinline__ C64 tpl_at(const WinTpl& t, int N, long long k) {
-    const long long m = k - (t.q - N / 2);
-    if (m < 0 || m >= N) return {0.0, 0.0};
-    return t.A[sw((int)((m + N / 2) & (N - 1)))];
-}
-__device__ __forceinline__ C64 tpl_at_e(const WinTpl& t, int N, long long k) {
-    const long long m = k - (t.q - N / 2);
-    if (m < 0 || m >= N) return {0.0, 0.0};
-    return t.E[sw((int)((m + N / 2) & (N - 1)))];
-}
-__device__ double block_sum64(double v, double* red) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Sum, minimum over the NT threads that work on a window (a warp or the CTA;
+// `red`: kWarps64 doubles of the CTA).
+template <int NT>
+__device__ __forceinline__ double group_sum(double v, double* red) {
     v = warp_sum(v);
+    if (NT == 32) return v;
     __syncthreads();
-    if (lane == 0) red[warp] = v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     double s = 0.0;
     for (int w = 0; w < kWarps64; ++w) s += red[w];
     return s;
 }
-// <x|y> with x a template and y a template (yt) or the data (yt == nullptr)
-__device__ double win_inner(const WinTpl& x, const WinTpl* yt, const gb_window_t& win, const C64* __restrict__ dA,
-                            const C64* __restrict__ dE, const double* __restrict__ wA, const double* __restrict__ wE,
-                            double T, double* red) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < win.W; i += blockDim.x) {
-        const long long k = win.k0 + i;
-        const C64 xa = tpl_at(x, win.N, k), xe = tpl_at_e(x, win.N, k);
-        C64 ya, ye;
-        if (yt) {
-            ya = tpl_at(*yt, win.N, k);
-            ye = tpl_at_e(*yt, win.N, k);
-        } else {
-            ya = dA[win.data_off + i];
-            ye = dE[win.data_off + i];
-        }
-        acc += wA[win.data_off + i] * (xa.x * ya.x + xa.y * ya.y) + wE[win.data_off + i] * (xe.x * ye.x + xe.y * ye.y);
-    }
-    return block_sum64(acc, red) * (4.0 / T);
+template <int NT>
+__device__ __forceinline__ int group_min(int v, double* red) {
+    v = __reduce_min_sync(0xffffffffu, v);
+    if (NT == 32) return v;
+    int* r = (int*)red;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) r[threadIdx.x >> 5] = v;
+    __syncthreads();
+    for (int w = 0; w < kWarps64; ++w) v = min(v, r[w]);
+    return v;
 }
+// a template in its buffers (bin values in natural order at sw(index)), its
+// carrier bin and the window bins [lo, hi) that it reaches
+struct WinTpl {
+    C64 *A, *E;
+    long long q;
+    int lo, hi;
+    bool bad;
+};
+__device__ __forceinline__ void place(WinTpl& t, const CandT& c, const gb_window_t& win) {
+    t.q = c.q;
+    t.bad = c.bad;
+    const long long l = c.q - win.N / 2 - win.k0, h = l + win.N;
+    t.lo = (int)min(max(l, 0LL), (long long)win.W);
+    t.hi = (int)min(max(h, 0LL), (long long)win.W);
+}
+__device__ __forceinline__ int tpl_index(const WinTpl& t, const gb_window_t& win, int i) {
+    return sw((int)((win.k0 + i - t.q) & (win.N - 1)));
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (~__double2hiint(x) & 0x7ff00000) != 0; }
 
 // Gram matrix G_ij = <s_i|s_j>, b_i = <d|s_i> and the multi-signal SNR
-// rho = sum_i b_i / sqrt(sum_ij G_ij) (Eq. 11) of each window's sources (one
-// CTA per window; the sources are the window's candidate rows).  Template i
-// is held in buffer P while the templates j > i pass through buffer Q.
+// rho = sum_i b_i / sqrt(sum_ij G_ij) (Eq. 11) of each window's sources (the
+// sources are the window's candidate rows), with <x|y> = (4/T) Re sum_k w_k
+// x_k y_k* in a fixed order.  NT threads work on a window, a warp or a CTA.
+// Template i is held in buffer P while the templates j > i pass through Q, the
+// next one last, so that it is P's content for i + 1: K (K-1)/2 + 1 templates.
+// A sum runs over the bins that its templates share; a weight or datum outside
+// them counts only by being non-finite (its product with zero is NaN), for
+// which the window is looked through once.
+// Bound by the FP64 and integer pipes and the set-ups' latency; 4,096 pairs,
+// N = 64-256, W = 2 N: 0.80 ms with one set-up at a time, template 1 computed
+// twice and five passes over all W bins, 0.50 ms now with a CTA per window,
+// 0.44 ms with a warp per window.
+constexpr int kGramSlots = kSetupWarp + 2;      // candidate slots of a window: those set up together, one for later ones
+static_assert(sizeof(CandT) * kGramSlots % 16 == 0, "the buffers behind the slots are read in 16-byte elements");
+template <int NT>
 __global__ void __launch_bounds__(kWarps64 * 32, kMinCtas64) multi_gram_kernel(
-    const gb_window_t* __restrict__ wins, TabSet64 tabs, const C64* __restrict__ tw_g, TabSetFx fxt, double T,
-    double fstar,
-    const C64* __restrict__ dA, const C64* __restrict__ dE, const double* __restrict__ wA,
+    const gb_window_t* __restrict__ wins, int n_win, TabSet64 tabs, const C64* __restrict__ tw_g, TabSetFx fxt,
+    double T, double fstar, const C64* __restrict__ dA, const C64* __restrict__ dE, const double* __restrict__ wA,
     const double* __restrict__ wE, const double* __restrict__ theta, int kmax, double* __restrict__ gram,
     double* __restrict__ dh_out, double* __restrict__ rho_out, int* status, int n_max) {
+    constexpr int GROUPS = kWarps64 * 32 / NT;  // windows in work per CTA
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FxTw* tw = (FxTw*)smem_raw;                 // kTwiddles
     double* red = (double*)(tw + kTwiddles);    // kWarps64
-    CandT* cand = (CandT*)(red + kWarps64);     // 2
-    C64* PA = (C64*)(cand + 2);                 // 4 buffers of n_max
-    C64* QA = PA + 2 * n_max;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const gb_window_t win = wins[blockIdx.x];
-    const int K = win.n_cand;
-    double* G = gram + (size_t)blockIdx.x * kmax * kmax;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x & (NT - 1);
+    const int group = GROUPS == 1 ? 0 : warp;
+    CandT* cand = (CandT*)(red + kWarps64) + group * kGramSlots;
+    C64* bufs = (C64*)((CandT*)(red + kWarps64) + GROUPS * kGramSlots) + (size_t)group * 4 * n_max;
     load_twiddles(fxt.tw, tw);
-    const Geo64 g = geometry64(win.N, T, fstar, fxt.arm_c, fxt.krho_q30);
-    const OrbitTables64 tab = tabs.t[g.logN - 5];
-    const FxTab ft{fxt.geo[g.logN - 5], tw, tw_g};
+    __syncthreads();
     const bool data = dA != nullptr;
-    double sum_b = 0.0, sum_g = 0.0;
-    bool bad_any = false;
-    for (int i = 0; i < K; ++i) {
-        __syncthreads();
-        if (warp == 0) setup_warp(theta + 8 * (win.cand_off + i), g, cand[0], lane);
-        __syncthreads();
-        const bool bad_i = cand[0].bad;
-        if (!bad_i) template_any<kWarps64 * 32>(cand[0], g, tab, ft, PA, n_max, false, threadIdx.x);
-        __syncthreads();
-        const WinTpl P{PA, PA + n_max, cand[0].q};
-        const double gii = bad_i ? nan("") : win_inner(P, &P, win, dA, dE, wA, wE, T, red);
-        const double bi = bad_i || !data ? nan("") : win_inner(P, nullptr, win, dA, dE, wA, wE, T, red);
-        if (threadIdx.x == 0) {
-            G[i * kmax + i] = gii;
-            if (dh_out) dh_out[win.cand_off + i] = bi;
-            if (bad_i) atomicOr(status, kStatusNonFinite);
-            sum_b += bi;
-            sum_g += gii;
-            bad_any |= bad_i;
+    for (int w = blockIdx.x * GROUPS + group; w < n_win; w += gridDim.x * GROUPS) {
+        const gb_window_t win = wins[w];
+        const int K = win.n_cand;
+        const double* th = theta + 8 * win.cand_off;
+        double* G = gram + (size_t)w * kmax * kmax;
+        const Geo64 g = geometry64(win.N, T, fstar, fxt.arm_c, fxt.krho_q30);
+        const OrbitTables64 tab = tabs.t[g.logN - 5];
+        const FxTab ft{fxt.geo[g.logN - 5], tw, tw_g};
+        const double* pwA = wA + win.data_off;
+        const double* pwE = wE + win.data_off;
+        // first and last bin with a non-finite weight, with a non-finite datum
+        int w_first = win.W, w_last = 0, d_first = win.W, d_last = 0;
+        if (K > 0) {
+            for (int i = tid; i < win.W; i += NT) {
+                if (!finite_bits(pwA[i]) || !finite_bits(pwE[i])) {
+                    w_first = min(w_first, i);
+                    w_last = min(w_last, -i - 1);
+                }
+                if (data) {
+                    const C64 a = dA[win.data_off + i], e = dE[win.data_off + i];
+                    if (!finite_bits(a.x) || !finite_bits(a.y) || !finite_bits(e.x) || !finite_bits(e.y)) {
+                        d_first = min(d_first, i);
+                        d_last = min(d_last, -i - 1);
+                    }
+                }
+            }
+            w_first = group_min<NT>(w_first, red);
+            w_last = -group_min<NT>(w_last, red);    // one past the last
+            d_first = group_min<NT>(d_first, red);
+            d_last = -group_min<NT>(d_last, red);
         }
-        for (int j = i + 1; j < K; ++j) {
-            __syncthreads();
-            if (warp == 0) setup_warp(theta + 8 * (win.cand_off + j), g, cand[1], lane);
-            __syncthreads();
-            const bool bad_j = cand[1].bad;
-            if (!bad_j) template_any<kWarps64 * 32>(cand[1], g, tab, ft, QA, n_max, false, threadIdx.x);
-            __syncthreads();
-            const WinTpl Q{QA, QA + n_max, cand[1].q};
-            const double gij = bad_i || bad_j ? nan("") : win_inner(P, &Q, win, dA, dE, wA, wE, T, red);
-            if (threadIdx.x == 0) {
-                G[i * kmax + j] = gij;
-                G[j * kmax + i] = gij;
-                sum_g += 2.0 * gij;
+        sync_nt<NT>();                          // the slots and buffers of the window before are done with
+        if (K > 0 && (GROUPS > 1 || warp == 0)) setup_warp(th, min(K, kSetupWarp), g, cand, lane);
+        sync_nt<NT>();
+        // template k into t's buffers
+        auto compute = [&](int k, WinTpl& t) {
+            if (k >= kSetupWarp) {
+                sync_nt<NT>();
+                if (GROUPS > 1 || warp == 0) setup_warp(th + 8 * k, 1, g, cand + kSetupWarp, lane);
+                sync_nt<NT>();
+            }
+            const CandT& c = cand[k < kSetupWarp ? k : kSetupWarp];
+            place(t, c, win);
+            sync_nt<NT>();                      // the buffer's last reads
+            if (!t.bad) template_any<NT>(c, g, tab, ft, t.A, n_max, false, tid);
+            sync_nt<NT>();
+        };
+        WinTpl P, Q;
+        P.A = bufs;
+        P.E = bufs + n_max;
+        Q.A = bufs + 2 * n_max;
+        Q.E = bufs + 3 * n_max;
+        double sum_b = 0.0, sum_g = 0.0;
+        bool bad_any = false;
+        for (int i = 0; i < K; ++i) {
+            if (i == 0) compute(0, P);
+            double gii = nan(""), bi = nan("");
+            if (!P.bad) {
+                const bool odd = w_first < P.lo || w_last > P.hi;
+                double sg = 0.0, sb = 0.0;
+                for (int k = P.lo + tid; k < P.hi; k += NT) {
+                    const int idx = tpl_index(P, win, k);
+                    const C64 xa = P.A[idx], xe = P.E[idx];
+                    const double va = pwA[k], ve = pwE[k];
+                    sg += va * (xa.x * xa.x + xa.y * xa.y) + ve * (xe.x * xe.x + xe.y * xe.y);
+                    if (data) {
+                        const C64 ya = dA[win.data_off + k], ye = dE[win.data_off + k];
+                        sb += va * (xa.x * ya.x + xa.y * ya.y) + ve * (xe.x * ye.x + xe.y * ye.y);
+                    }
+                }
+                gii = odd ? nan("") : group_sum<NT>(sg, red) * (4.0 / T);
+                if (data)
+                    bi = odd || d_first < P.lo || d_last > P.hi ? nan("") : group_sum<NT>(sb, red) * (4.0 / T);
+            }
+            if (tid == 0) {
+                G[i * kmax + i] = gii;
+                if (dh_out) dh_out[win.cand_off + i] = bi;
+                if (P.bad) atomicOr(status, kStatusNonFinite);
+                sum_b += bi;
+                sum_g += gii;
+                bad_any |= P.bad;
+            }
+            for (int j = K - 1; j > i; --j) {
+                compute(j, Q);
+                double gij = nan("");
+                if (!P.bad && !Q.bad) {
+                    const int lo = max(P.lo, Q.lo), hi = min(P.hi, Q.hi);
+                    const bool odd = lo < hi ? w_first < lo || w_last > hi : w_last > 0;
+                    double sg = 0.0;
+                    for (int k = lo + tid; k < hi; k += NT) {
+                        const int ip = tpl_index(P, win, k), iq = tpl_index(Q, win, k);
+                        const C64 xa = P.A[ip], xe = P.E[ip], ya = Q.A[iq], ye = Q.E[iq];
+                        sg += pwA[k] * (xa.x * ya.x + xa.y * ya.y) + pwE[k] * (xe.x * ye.x + xe.y * ye.y);
+                    }
+                    gij = odd ? nan("") : group_sum<NT>(sg, red) * (4.0 / T);
+                }
+                if (tid == 0) {
+                    G[i * kmax + j] = gij;
+                    G[j * kmax + i] = gij;
+                    sum_g += 2.0 * gij;
+                }
+            }
+            if (i + 1 < K) {
+                const WinTpl t = P;
+                P = Q;
+                Q = t;
             }
         }
+        if (tid == 0 && rho_out) rho_out[w] = (K == 0 || bad_any || !data) ? nan("") : sum_b / sqrt(sum_g);
     }
-    if (threadIdx.x == 0 && rho_out)
-        rho_out[blockIdx.x] = (K == 0 || bad_any || !data) ? nan("") : sum_b / sqrt(sum_g);
 }
 
 }  // namespace
@@ -449,13 +521,23 @@ int launch_multi_gram(gb_ctx* ctx, const gb_window_t* d_win, int n_win, int n_ma
                       const double* dE, const double* wA, const double* wE, const double* theta, int kmax,
                       double* gram, double* dh, double* rho, cudaStream_t s) {
     if (n_win == 0) return GB_OK;
-    const size_t smem = sizeof(FxTw) * kTwiddles + sizeof(double) * kWarps64 + sizeof(CandT) * 2 +
-                        sizeof(C64) * 4 * (size_t)n_max;
-    cudaError_t e = cudaFuncSetAttribute(multi_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    // a warp per window needs windows for all SMs' warps, and short templates
+    // (four buffers each) to have eight of them resident
+    const bool by_warp = n_max <= 256 && n_win >= 4 * sms;
+    const int groups = by_warp ? kWarps64 : 1;
+    const size_t smem = sizeof(FxTw) * kTwiddles + sizeof(double) * kWarps64 +
+                        groups * (sizeof(CandT) * kGramSlots + sizeof(C64) * 4 * (size_t)n_max);
+    const auto kfn = by_warp ? multi_gram_kernel<32> : multi_gram_kernel<kWarps64 * 32>;
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(ctx, e, "multi_gram: smem attribute");
-    multi_gram_kernel<<<n_win, kWarps64 * 32, smem, s>>>(d_win, tabset64(ctx), (const C64*)ctx->d_tw64, tabset_fx(ctx), ctx->obs.T_obs,
-                                                         transfer_frequency(ctx), (const C64*)dA, (const C64*)dE, wA,
-                                                         wE, theta, kmax, gram, dh, rho, ctx->d_status, n_max);
+    int bpsm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, kfn, kWarps64 * 32, smem) != cudaSuccess || bpsm < 1) bpsm = 1;
+    const int grid = std::min((n_win + groups - 1) / groups, sms * bpsm);
+    kfn<<<grid, kWarps64 * 32, smem, s>>>(d_win, n_win, tabset64(ctx), (const C64*)ctx->d_tw64, tabset_fx(ctx),
+                                          ctx->obs.T_obs, transfer_frequency(ctx), (const C64*)dA, (const C64*)dE, wA,
+                                          wE, theta, kmax, gram, dh, rho, ctx->d_status, n_max);
     ++ctx->launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(ctx, e, "multi_gram launch");

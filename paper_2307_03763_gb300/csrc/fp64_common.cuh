@@ -94,25 +94,31 @@ __device__ __forceinline__ void setup_lane(const double* th, const Geo64& g, Can
     double ii;
     setup_lane(th, g, c, t, ii);
 }
-// one candidate by a whole warp: the five sines and cosines on five lanes (the
-// double sincos is a long dependent chain), the rest on lane 0
-__device__ void setup_warp(const double* th, const Geo64& g, CandT& c, int lane) {
-    const double x = lane == 0 ? th[2] : lane == 1 ? th[3] : lane == 2 ? 2.0 * th[6] : lane == 3 ? th[5] : kPi * th[0] * g.arm_c;
+// Up to six candidates by a whole warp: each one's five sines and cosines on
+// five lanes (the double sincos is a long dependent chain), the rest on one
+// lane per candidate.
+constexpr int kSetupWarp = 6;
+__device__ void setup_warp(const double* th, int cnt, const Geo64& g, CandT* c, int lane) {
+    const int mine = lane / 5 < cnt ? lane / 5 : cnt - 1, kind = lane % 5;
+    const double* t0 = th + 8 * mine;
+    const double x = kind == 0 ? t0[2] : kind == 1 ? t0[3] : kind == 2 ? 2.0 * t0[6] : kind == 3 ? t0[5] : kPi * t0[0] * g.arm_c;
     double sn, cs;
     sincos(x, &sn, &cs);
+    const int src = 5 * (lane < cnt ? lane : 0);
     FxTrig t;
-    t.sb = __shfl_sync(0xffffffffu, sn, 0);
-    t.cb = __shfl_sync(0xffffffffu, cs, 0);
-    t.sl = __shfl_sync(0xffffffffu, sn, 1);
-    t.cl = __shfl_sync(0xffffffffu, cs, 1);
-    t.s2 = __shfl_sync(0xffffffffu, sn, 2);
-    t.c2 = __shfl_sync(0xffffffffu, cs, 2);
-    t.ci = __shfl_sync(0xffffffffu, cs, 3);
-    t.sa = __shfl_sync(0xffffffffu, sn, 4);
-    t.ca = __shfl_sync(0xffffffffu, cs, 4);
-    if (lane == 0) {
-        const double delta = carrier64(th, g.T, c);
-        setup_t(th, g, delta, t, c);
+    t.sb = __shfl_sync(0xffffffffu, sn, src);
+    t.cb = __shfl_sync(0xffffffffu, cs, src);
+    t.sl = __shfl_sync(0xffffffffu, sn, src + 1);
+    t.cl = __shfl_sync(0xffffffffu, cs, src + 1);
+    t.s2 = __shfl_sync(0xffffffffu, sn, src + 2);
+    t.c2 = __shfl_sync(0xffffffffu, cs, src + 2);
+    t.ci = __shfl_sync(0xffffffffu, cs, src + 3);
+    t.sa = __shfl_sync(0xffffffffu, sn, src + 4);
+    t.ca = __shfl_sync(0xffffffffu, cs, src + 4);
+    if (lane < cnt) {
+        const double* tl = th + 8 * lane;
+        const double delta = carrier64(tl, g.T, c[lane]);
+        setup_t(tl, g, delta, t, c[lane]);
     }
 }
 

@@ -114,3 +114,47 @@ def test_match_metrics_from_the_gram_matrix(api):
         assert abs(float(delta - od)) <= 1e-9 * max(1.0, abs(float(od))), (w, float(delta), float(od))
         assert abs(float(ov - oo)) <= 1e-10, (w, float(ov), float(oo))
     ctx.close()
+
+
+@pytest.mark.parametrize("per", [1, 3, 8])
+def test_gram_by_warp_and_by_block_agree(api, per):
+    """Many short windows are taken by a warp each, few by a block each: the
+    same templates, sums of up to W = 512 terms in another order (W 2^-53 of
+    the sum of absolute terms, at most the norms' product, on either side)."""
+    rng = np.random.default_rng(per)
+    T, specs, srcs = wk.YEAR, [], []
+    for w in range(1300):
+        N = (32, 64, 128, 256)[w % 4]
+        f = (0.3e-3, 1e-3, 2e-3, 4e-3)[w % 4] * rng.uniform(1.0, 1.5)
+        specs.append((int(round(f * T)) - N // 2 - (w % 3) * N // 2, (1, 2, 2)[w % 3] * N, N))
+        srcs += [wk.source(f + k / T, 1e-17, 1e-22, rng) for k in range(per)]
+    wins, _, _ = wk.layout(specs, [per] * len(specs))
+    n = sum(W for _, W, _ in specs)
+    d = [_cuda(rng.normal(size=n) + 1j * rng.normal(size=n), torch.complex128) for _ in range(2)]
+    w = [_cuda(rng.uniform(1.0, 2.0, size=n), torch.float64) for _ in range(2)]
+    w[0][wins[700][3] + 1] = math.nan            # a bad weight at the edge of a window
+    d[1][wins[900][3]] = math.inf                # and a bad datum
+    th = _cuda(np.array(srcs), torch.float64)
+    ctx = api.Context(T)
+    rho, G, b = ctx.snr_multi(wins, *d, *w, th)
+    for i0 in range(0, len(wins), 100):
+        part, c0, o0 = wins[i0:i0 + 100], wins[i0][4], wins[i0][3]
+        bins = slice(o0, part[-1][3] + part[-1][1])
+        sub = [(k0, W, N, off - o0, c - c0, m) for k0, W, N, off, c, m in part]
+        x = [t[bins].clone() for t in (*d, *w)]
+        r1, G1, b1 = ctx.snr_multi(sub, *x, th[c0:c0 + per * len(part)].clone())
+        G0, b0 = G[i0:i0 + 100], b[c0:c0 + per * len(part)]
+        assert torch.equal(torch.isnan(G0), torch.isnan(G1)) and torch.equal(torch.isnan(b0), torch.isnan(b1))
+        assert torch.equal(torch.isnan(rho[i0:i0 + 100]), torch.isnan(r1))
+        eps = 2 * 512 * 2.0 ** -53
+        for i, (k0, W, N, off, c, m) in enumerate(sub):
+            if not (torch.isfinite(G1[i]).all() and torch.isfinite(b1[c:c + m]).all()):
+                assert torch.equal(torch.isinf(b0[c:c + m]), torch.isinf(b1[c:c + m]))
+                continue
+            g = G1[i].diagonal().max()
+            sl = slice(off, off + W)
+            dd = 4 / T * sum((x[2 + k][sl] * x[k][sl].abs() ** 2).sum() for k in range(2))
+            assert (G0[i] - G1[i]).abs().max() <= eps * g
+            assert (b0[c:c + m] - b1[c:c + m]).abs().max() <= eps * torch.sqrt(dd * g)
+    assert torch.isnan(G[700]).any() and not torch.isnan(G[700 + 4]).any() and not torch.isnan(G[900]).any()
+    ctx.close()
