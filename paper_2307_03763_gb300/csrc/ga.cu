@@ -90,6 +90,38 @@ __device__ __forceinline__ double wrap(double x, double lo, double hi) {
     return lo + y;
 }
 
+// A float as a double, by its bits: the conversion instruction runs on the FP64
+// pipe, 64 clocks per warp.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    if ((b & 0x7f800000u) == 0u) return (double)f;   // zero, subnormal
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// A double's bits in the order of the numbers, -0 below +0
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// (float)hypot(a, b), the same bits: the root of a^2 + b^2 in float with one
+// correction, good to 2^-46, rounded once; hypot itself where that is too near
+// a tie, at a power of two or out of float's range.
+__device__ __forceinline__ float hypot_float(double a, double b) {
+    const double r2 = fma(a, a, b * b);
+    const float q = (float)r2;
+    if (q > 1e-30f && q < 1e30f) {
+        const float s = sqrtf(q);
+        const double sd = widen(s);
+        const float c = (float)fma(-sd, sd, r2) / (2.0f * s);
+        const float r = __fadd_rn(s, c), rest = __fsub_rn(c, __fsub_rn(r, s));
+        const uint32_t rb = __float_as_uint(r);
+        const float h = __uint_as_float((rb & 0x7f800000u) - (24u << 23));   // half an ulp of r
+        if ((rb & 0x7fffffu) != 0u && fabsf(fabsf(rest) - h) > h * 0x1p-15f) return r;
+    }
+    return (float)hypot(a, b);
+}
+
 // rho = <d|h>/sqrt(<h|h>) (Eq. 6), in float: it only ranks individuals
 __device__ __forceinline__ float fitness(double dh, double hh) {
     if (!(hh > 0.0) || !isfinite(dh) || !isfinite(hh)) return -INFINITY;
@@ -98,7 +130,49 @@ __device__ __forceinline__ float fitness(double dh, double hh) {
     return (float)(dh / sqrt(hh));
 }
 
-__global__ void __launch_bounds__(kGaThreads) ga_step_kernel(int pop, const double* __restrict__ theta,
+// fitness(dh, hh) and fitness(hypot(dh, di), hh), with the range tests in float
+__device__ __forceinline__ float fitness_fast(double dh, double hh) {
+    const float h = (float)hh, d = (float)dh;
+    if (h >= 1e-30f && h <= 1e30f && fabsf(d) < 1e29f) return d * rsqrtf(h);
+    return fitness(dh, hh);
+}
+__device__ __forceinline__ float fitness_fast(double dh, double di, double hh) {
+    const float h = (float)hh, d = hypot_float(dh, di);
+    if (h >= 1e-30f && h <= 1e30f && d < 1e29f) return d * rsqrtf(h);
+    return fitness(hypot(dh, di), hh);
+}
+
+// A row of eight doubles; wide: its address is a multiple of 16 bytes
+__device__ __forceinline__ void load_row(const double* p, bool wide, double (&v)[8]) {
+    if (wide) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const double2 x = ((const double2*)p)[j];
+            v[2 * j] = x.x;
+            v[2 * j + 1] = x.y;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = p[j];
+    }
+}
+__device__ __forceinline__ void store_row(double* p, bool wide, const double (&v)[8]) {
+    if (wide) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ((double2*)p)[j] = make_double2(v[2 * j], v[2 * j + 1]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) p[j] = v[j];
+    }
+}
+
+// Bound by the FP64 pipe (64 clocks per warp instruction): what only ranks,
+// tests or converts is done with integers and floats, with the same results.
+// 1,200 populations of 1,024: 0.36 ms before, 0.24 ms now.  The draws of the
+// eight parameters are a loop, not unrolled, under a register cap that lets
+// eight blocks share an SM (unrolled, 2 blocks: 0.33 ms; a loop, 3, 4 or 6
+// blocks: 0.28, 0.25, 0.26).
+__global__ void __launch_bounds__(kGaThreads, 8) ga_step_kernel(int pop, const double* __restrict__ theta,
                                                              const double* __restrict__ dh,
                                                              const double* __restrict__ hh,
                                                              const double* __restrict__ dh_im,
@@ -111,6 +185,17 @@ __global__ void __launch_bounds__(kGaThreads) ga_step_kernel(int pop, const doub
     __shared__ float s_fit[kGaThreads];
     __shared__ int s_idx[kGaThreads];
     __shared__ double s_best[8];
+    __shared__ long long s_lo[8], s_hi[8];   // keys of the box: a value with s_lo <= key <= s_hi is inside
+    if (threadIdx.x < 8) {
+        const int j = threadIdx.x;
+        const double lo = box[blockIdx.x].lo[j], hi = box[blockIdx.x].hi[j];
+        const bool wraps = j == 3 || j == 6 || j == 7;
+        // wrapped parameters: strictly below hi (below -0 where hi is 0); no
+        // value passes a bound that is not a number
+        const bool ok = lo == lo && hi == hi;
+        s_lo[j] = ok ? order_key(lo) : 0x7fffffffffffffffLL;
+        s_hi[j] = !ok ? -0x7fffffffffffffffLL - 1 : !wraps ? order_key(hi) : order_key(hi == 0.0 ? -0.0 : hi) - 1;
+    }
     const int w = blockIdx.x;
     const uint64_t generation = *gen_in;
     if (w == 0 && threadIdx.x == 0) *gen_out = generation + 1;
@@ -124,8 +209,8 @@ __global__ void __launch_bounds__(kGaThreads) ga_step_kernel(int pop, const doub
     float bf = -INFINITY;
     int bi = 0;
     for (int i = threadIdx.x; i < pop; i += blockDim.x) {
-        const float f = pmax ? fitness(hypot(dh[base + i], dh_im[base + i]), hh[base + i])
-                             : fitness(dh[base + i], hh[base + i]);
+        const float f = pmax ? fitness_fast(dh[base + i], dh_im[base + i], hh[base + i])
+                             : fitness_fast(dh[base + i], hh[base + i]);
         s_pop_fit[i] = f;
         if (f > bf) {
             bf = f;
@@ -172,6 +257,7 @@ __global__ void __launch_bounds__(kGaThreads) ga_step_kernel(int pop, const doub
         }
         gnorm = sqrt(gnorm);
     }
+    const bool wide_in = ((size_t)theta & 15) == 0, wide_out = ((size_t)out & 15) == 0;
     bool all_c, all_m;
     const uint32_t thr_c = prob_threshold(prm.p_cross, all_c), thr_m = prob_threshold(prm.p_mut, all_m);
     double sigma[8];
@@ -202,24 +288,27 @@ __global__ void __launch_bounds__(kGaThreads) ga_step_kernel(int pop, const doub
                 }
                 par[p] = win_i;
             }
+            double pa[8], pb[8];
+            load_row(th + 8 * par[0], wide_in, pa);
+            load_row(th + 8 * par[1], wide_in, pb);
+#pragma unroll 1
             for (int j = 0; j < 8; ++j) {
-                const double a = th[8 * par[0] + j], b = th[8 * par[1] + j];
-                const double t = (double)rng.uniform_f();
+                const double a = pa[j], b = pb[j];
+                const double t = widen(rng.uniform_f());
                 double x = rng.bernoulli(thr_c, all_c) ? fma(t, b - a, a) : a;
-                if (rng.bernoulli(thr_m, all_m)) x = fma(sigma[j], (double)rng.normal_f(), x);
+                if (rng.bernoulli(thr_m, all_m)) x = fma(sigma[j], widen(rng.normal_f()), x);
                 c[j] = x;
             }
         }
         // back into the prior box
-        c[0] = reflect(c[0], bx.lo[0], bx.hi[0]);
-        c[1] = reflect(c[1], bx.lo[1], bx.hi[1]);
-        c[2] = reflect(c[2], bx.lo[2], bx.hi[2]);
-        c[3] = wrap(c[3], bx.lo[3], bx.hi[3]);
-        c[4] = reflect(c[4], bx.lo[4], bx.hi[4]);
-        c[5] = reflect(c[5], bx.lo[5], bx.hi[5]);
-        c[6] = wrap(c[6], bx.lo[6], bx.hi[6]);
-        c[7] = wrap(c[7], bx.lo[7], bx.hi[7]);
-        for (int j = 0; j < 8; ++j) to[8 * i + j] = c[j];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const long long k = order_key(c[j]);
+            if (k >= s_lo[j] && k <= s_hi[j]) continue;
+            const bool wraps = j == 3 || j == 6 || j == 7;
+            c[j] = wraps ? wrap(c[j], bx.lo[j], bx.hi[j]) : reflect(c[j], bx.lo[j], bx.hi[j]);
+        }
+        store_row(to + 8 * i, wide_out, c);
     }
 }
 

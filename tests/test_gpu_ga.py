@@ -308,3 +308,56 @@ def test_newton_polish_reaches_the_maximum(api):
     # (A, iota, psi, phi0) move along their curved degeneracy valley
     assert float(L[0]) > max(float(l0[0]), -0.1), (float(l0[0]), float(L[0]))
     assert np.all(np.abs(th[:4] - src[:4]) < 0.05 * sig[:4]), (th - src) / sig
+
+
+@pytest.mark.parametrize("phase", [False, True])
+@pytest.mark.parametrize("pop", [1, 31, 700])
+def test_step_on_any_alignment_and_range(api, phase, pop):
+    """Rows on and off a 16-byte boundary give the same bits; the best
+    individual is the one of largest rho over values inside and outside
+    float's range (no-number, infinite and non-positive ones rank last);
+    selection without crossover and mutation returns rows of the population
+    folded into the box, also at bounds of zero."""
+    rng = np.random.default_rng(pop)
+    n_win, T = 5, wk.YEAR
+    n = n_win * pop
+    th = rng.uniform(-1.0, 1.0, (n, 8))
+    th[::7, :] = 0.0
+    th[::11, :] = -0.0
+    box = np.zeros((n_win, 16))
+    box[:, :8], box[:, 8:] = -1.0, 1.0
+    box[:, 7], box[:, 15] = 0.0, 2 * math.pi              # the whole circle: the phase may be maximised
+    box[1, 8:15] = 0.0                                    # upper bounds of zero
+    box[2, :7] = -0.0
+    scale = np.exp(rng.uniform(-200.0, 200.0, n)) if pop == 700 else np.exp(rng.uniform(-20.0, 20.0, n))
+    dh, di = rng.normal(size=n) * scale, rng.normal(size=n) * scale
+    hh = scale ** 2 * np.exp(rng.uniform(-3.0, 3.0, n))
+    dh[3::50], hh[5::50], hh[7::50], hh[9::50] = np.nan, 0.0, np.inf, -1.0
+    with np.errstate(all="ignore"):
+        num = np.hypot(dh, di) if phase else dh
+        rho = np.where((hh > 0) & np.isfinite(hh) & np.isfinite(num), num / np.sqrt(hh), -np.inf).reshape(n_win, pop)
+    ctx = api.Context(T)
+    prm = api.GAParams(3, 0, 0.0, 0.0, 0.1)
+    gen, nxt = torch.zeros(1, dtype=torch.int64, device=DEV), torch.zeros(1, dtype=torch.int64, device=DEV)
+    res = []
+    for off in (0, 1):
+        def at(x):
+            t = torch.empty(x.size + 1, dtype=torch.float64, device=DEV)[off:off + x.size].view(x.shape)
+            t.copy_(torch.as_tensor(x))
+            return t
+        out = at(np.zeros_like(th))
+        _, best = ctx.ga_step(n_win, pop, at(th), at(dh), at(hh), at(box), 5, gen, nxt, prm, out=out,
+                              dh_im=at(di) if phase else None)
+        res.append((out.clone(), best.clone()))
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
+    out, best = (x.cpu().numpy() for x in res[0])
+    th, out = th.reshape(n_win, pop, 8), out.reshape(n_win, pop, 8)
+    for w in range(n_win):
+        if np.isfinite(rho[w]).any():
+            top = np.sort(rho[w])[::-1]
+            if pop == 1 or top[1] < top[0] * (1 - 1e-5):
+                assert np.array_equal(best[w, :4], th[w, rho[w].argmax(), :4])
+    for w in (0, 3, 4):                                   # nothing to fold in parameters 0 .. 6
+        rows = {r.tobytes() for r in th[w, :, :7] + 0.0}
+        assert all((r + 0.0).tobytes() in rows for r in out[w, 1:, :7])
+    assert (out[1, 1:, :7] <= 0.0).all() and (out[2, 1:, :7] >= 0.0).all()
