@@ -174,7 +174,9 @@ __global__ void __cluster_dims__(kKdeCtas, 1, 1) __launch_bounds__(kKdeThreads)
         red[3][warp] = by_;
         redc[warp] = acc;
     }
-    __syncthreads();
+    // a CTA's shared memory may be reached only once it runs: no remote store
+    // before this barrier (behind the gathers, whose latency hides it)
+    cl.sync();
     // ordered sums: x in warp 0, y in warp 1; range and moves in warp 2
     if (warp < 2) {
         double s = 0.0;
@@ -492,8 +494,9 @@ extern "C" int gb_kde_build(gb_ctx_t* ctx, int32_t n_win, int32_t n, const doubl
     if (!theta || !chain || !box || !cdf || !ext) return set_error(ctx, GB_EINVAL, "gb_kde_build: null pointer");
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_error(ctx, e, "gb_kde_build: cudaSetDevice");
-    // a chain's entries stay in shared memory when they fit (up to about 65,000
-    // per chain); longer chains are gathered again in each pass
+    // a chain's entries stay in shared memory when they fit beside the grid (up
+    // to 88,064 per chain at grid 64, 52,736 at grid 128); longer chains are
+    // gathered again in each pass
     const int store = kde_build_smem(grid, n, true) <= 200 * 1024;
     const size_t smem = kde_build_smem(grid, n, store != 0);
     e = cudaFuncSetAttribute(kde_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -72,6 +72,31 @@ def test_kde_build_matches_oracle(api, grid):
         assert np.all(np.diff(got[w], axis=1) > 0) and np.allclose(got[w][:, -1], 1.0, atol=1e-12)
 
 
+# a single entry, CTAs of the cluster without entries or with part of a warp,
+# counts around a round of the cluster's 256; rows of the grid that do not
+# divide by its eight CTAs; chains whose entries do not fit in shared memory
+@pytest.mark.parametrize("n,grid", [(n, g) for n in (1, 31, 33, 255, 257, 1500) for g in (128, 13, 5)] +
+                         [(90000, 64), (55000, 128)])
+def test_kde_build_over_a_cluster(api, n, grid):
+    """Two smoothing passes of at most 2 grid fused float steps each, relative, in a cell and in the total."""
+    ctx = api.Context(wk.YEAR)
+    rng = np.random.default_rng(n + grid)
+    nw = 2
+    box = _boxes(rng, nw)
+    lo, hi = box[:, :8], box[:, 8:]
+    th = ((lo + hi) / 2)[:, None, :] + (hi - lo)[:, None, :] * rng.normal(0.0, 0.25, size=(nw, n, 8))
+    ch = _chains(rng, nw, n, [0.3, 0.02])
+    cdf = torch.empty((nw, 3, grid * grid), dtype=torch.float64, device=DEV)
+    ext = torch.empty((nw, 3, 4), dtype=torch.float64, device=DEV)
+    ctx.kde_build(_cuda(th.reshape(-1, 8), torch.float64), _cuda(ch, torch.int32), _cuda(box, torch.float64), grid,
+                  0.01, out=(cdf, ext))
+    got, gext = cdf.cpu().numpy(), ext.cpu().numpy()
+    for w in range(nw):
+        ref, rext = okde.build_window(th[w], ch[w], lo[w], hi[w], grid, 0.01)
+        assert np.allclose(gext[w], rext, rtol=1e-12, atol=0), (w, gext[w], rext)
+        assert np.abs(got[w] - ref).max() < 8 * grid * 2.0 ** -24, (w, np.abs(got[w] - ref).max())
+
+
 def test_kde_draw_matches_oracle(api):
     # tables from the oracle (one smoothed, one flat, one peaked), draws
     # compared proposal by proposal with the oracle fed the same Philox words
