@@ -119,7 +119,7 @@ int launch_loglik_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const d
         e = launch_mixed_part(kfn, grid, smem, s, plan.d_win, plan.d_meta, plan.d_prep, plan.d_tiles + first, n_items,
                               plan.d_head + part, tabset32(ctx), (const float2*)ctx->d_tw32, ctx->obs.T_obs,
                               transfer_frequency(ctx), theta, logL, dh, hh, dh_im, ctx->d_status, nmax,
-                              ctx->budget_ns, plan.n_prep, chain, dependent);
+                              ctx->budget_ns, plan.n_prep, chain == 0 ? kParts - 1 - part : -1, dependent);
         held = smem * bpsm;
         ++chain;
         ++ctx->launches;
@@ -387,7 +387,7 @@ extern "C" int gb_loglik_mixed_noalloc(const gb_obs_t* obs, const gb_window_t* w
         if (grid > need) grid = need;
         e = launch_mixed_part(kfn, grid, smem, s, d_win, d_meta, d_prep, d_items + first, n_items, d_head + part, tabs,
                               (const float2*)tw32, obs->T_obs, fstar, theta, logL, dh, hh, nullptr, d_status, nmax, 0ULL,
-                              0LL, chain, true);
+                              0LL, chain == 0 ? kParts - 1 - part : -1, true);
         ++chain;
         if (e == cudaSuccess) e = cudaGetLastError();
     }

@@ -1398,6 +1398,32 @@ __device__ __forceinline__ const U* after_wait(const U* p) {
     return p;
 }
 
+// Work queues of the parts, and how a later part sees the preparation's stores.
+// Only the wait makes them visible, and only to the kernel that waits: for a
+// later part that would be the end of the part before.  So the visibility is
+// handed on.  The preparation leaves every queue head closed; the chain's first
+// part, after its own wait and before it lets the next part start, opens the
+// later parts' heads (fence, then an atomic: a release), and a later
+// part's warp takes its first item by an atomic on its head followed by a fence
+// (an acquire).  A warp that met a closed head waits for the part before and
+// takes its item then; the opening has discarded its first attempt.
+constexpr int kQueueClosed = -(1 << 30);
+// (one thread) open the `later` heads after this part's own, those still closed
+__device__ __forceinline__ void open_queues(int* head, int later) {
+    __threadfence();
+    for (int p = 1; p <= later; ++p) atomicMax(head + p, 0);
+}
+// (one thread) the first item of a warp of a later part
+__device__ __forceinline__ int first_item_later(int* head) {
+    int item = atomicAdd(head, 1);
+    if (item < 0) {
+        pdl_wait();
+        item = atomicAdd(head, 1);
+    }
+    __threadfence();
+    return item;
+}
+
 // dT, wT (may be null): the T channel, used in windows whose lowest frequency
 // k0/T is at least f*/2; its float copy goes n_prep entries after A and E's.
 __global__ void prep_mixed_kernel(const gb_window_t* __restrict__ wins, WinMeta* __restrict__ meta,
@@ -1409,7 +1435,7 @@ __global__ void prep_mixed_kernel(const gb_window_t* __restrict__ wins, WinMeta*
     __shared__ double s_acc[32], s_max[32];
     pdl_launch_dependents();
     const int w = blockIdx.x;
-    if (w == 0 && threadIdx.x < kParts) head[threadIdx.x] = 0;   // the work queues
+    if (w == 0 && threadIdx.x < kParts) head[threadIdx.x] = kQueueClosed;   // the work queues
     const gb_window_t win = wins[w];
     const bool useT = dT != nullptr && (double)win.k0 / T >= 0.5 * fstar;
     double acc = 0.0, wmax = 0.0;
@@ -1493,7 +1519,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIX
     const Tile* __restrict__ items, int n_items, int* head, TabSet32 tabs, const float2* __restrict__ tw1024,
     double T, double fstar, const double* __restrict__ theta, double* __restrict__ logL,
     double* __restrict__ dh_out, double* __restrict__ hh_out, double* __restrict__ dhi_out, int* status, int n_max,
-    unsigned long long budget_ns, long long n_prep, int chain, int warp_bytes) {
+    unsigned long long budget_ns, long long n_prep, int later, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // per warp: the buffers of A and E, T's samples with T3 (one complex float
@@ -1508,12 +1534,13 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIX
     const double ifs = 1.0 / fstar;   // the float results do not see the reciprocal's rounding
 
     const unsigned long long t0 = budget_ns != 0ULL ? global_ns() : 0ULL;
-    // The chain's first part (chain 0) starts beside the preparation kernel:
-    // its warps' first items are fixed, and the queue hands out the others.
-    // Later parts start when the preparation is done, and take all from the queue.
-    const int fixed = chain == 0 ? (int)gridDim.x * kWarpsMx : 0;
-    bool waited = chain != 0;
-    if (waited) pdl_launch_dependents();
+    // The chain's first part (later: the queues after its own) starts beside
+    // the preparation kernel: its warps' first items are fixed, and the queue
+    // hands out the others.  Later parts (later < 0) start when the preparation
+    // is done, and take all from the queue.
+    const bool lead = later >= 0;
+    bool ready = false;   // the preparation's results are visible to this warp
+    if (!lead) pdl_launch_dependents();
     for (;;) {
         // a warp past the time budget takes no further item and flags it
         int item = blockIdx.x * kWarpsMx + warp;
@@ -1521,8 +1548,10 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIX
             if (budget_ns != 0ULL && global_ns() - t0 > budget_ns) {
                 atomicOr(status, kStatusBudget);
                 item = n_items;
-            } else if (waited) {
-                item = fixed + atomicAdd(head, 1);
+            } else if (!lead) {
+                item = ready ? atomicAdd(head, 1) : first_item_later(head);
+            } else if (ready) {
+                item = (int)gridDim.x * kWarpsMx - kQueueClosed + atomicAdd(head, 1);
             }
         }
         item = __shfl_sync(0xffffffffu, item, 0);
@@ -1534,10 +1563,14 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIX
         const int cnt = (int)(t.c_end - t.c_begin);
         if (lane < cnt) setup_mixed(theta + 8 * (t.c_begin + lane), T, ifs, cands[lane], N < 64);
         __syncwarp();
-        if (!waited) {
-            pdl_wait();
-            pdl_launch_dependents();
-            waited = true;
+        if (!ready) {
+            if (lead) {
+                // only after the wait and behind the opened queues may the next part start: its blocks rely on both
+                pdl_wait();
+                if (blockIdx.x == 0 && threadIdx.x == 0) open_queues(head, later);
+                pdl_launch_dependents();
+            }
+            ready = true;
         }
         const WinMeta wm = after_wait(meta)[t.win];
         const Win32* pw = after_wait(prep) + wm.prep_off;
@@ -1641,7 +1674,10 @@ __global__ void __launch_bounds__(kWarpsMx * 32, RMAX <= 8    ? (T3 ? 4 : GB_MIX
             }
         }
         __syncwarp();
-    }    pdl_wait();
+    }
+    pdl_wait();
+    // in case the first warp took no item (time budget)
+    if (lead && blockIdx.x == 0 && threadIdx.x == 0) open_queues(head, later);
 }
 
 int resident_blocks(const void* kernel, int threads, size_t smem) {
@@ -1685,10 +1721,10 @@ cudaError_t launch_mixed_part(const void* kfn, int grid, size_t smem, cudaStream
                               const WinMeta* meta, const Win32* prep, const Tile* items, int n_items, int* head,
                               TabSet32 tabs, const float2* tw1024, double T, double fstar, const double* theta,
                               double* logL, double* dh, double* hh, double* dhi, int* status, int n_max,
-                              unsigned long long budget_ns, long long n_prep, int chain, bool dependent) {
+                              unsigned long long budget_ns, long long n_prep, int later, bool dependent) {
     int warp_bytes = (int)(smem / kWarpsMx);
     void* args[] = {&wins, &meta, &prep, &items, &n_items, &head,  &tabs,      &tw1024, &T,     &fstar,
-                    &theta, &logL, &dh,  &hh,    &dhi,     &status, &n_max,    &budget_ns, &n_prep, &chain, &warp_bytes};
+                    &theta, &logL, &dh,  &hh,    &dhi,     &status, &n_max,    &budget_ns, &n_prep, &later, &warp_bytes};
     return launch_chained(kfn, grid, smem, s, args, dependent);
 }
 

@@ -41,10 +41,10 @@ int launch_grad_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const dou
         int* status = ctx->d_status;
         unsigned long long budget = ctx->budget_ns;
         long long n_prep = plan.n_prep;
-        int n_it = n_items, n_mx = nmax, warp_bytes = (int)(smem / kWarpsMx);
+        int n_it = n_items, n_mx = nmax, warp_bytes = (int)(smem / kWarpsMx), later = chain == 0 ? kParts - 1 - part : -1;
         void* args[] = {(void*)&plan.d_win, (void*)&plan.d_meta, (void*)&plan.d_prep, (void*)&items, &n_it, &head,
                         &tabs, &tw, &Tobs, &fstar, (void*)&theta, &logL, &grad, &status, &n_mx, &budget, &n_prep,
-                        &chain, &warp_bytes};
+                        &later, &warp_bytes};
         e = launch_chained(kfn, grid, smem, s, args, chain == 0 || held <= kHeldMax);
         held = smem * bpsm;
         ++chain;

@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel
     const Tile* __restrict__ items, int n_items, int* head, TabSet32 tabs, const float2* __restrict__ tw1024,
     double T, double fstar, const double* __restrict__ theta, double* __restrict__ logL,
     double* __restrict__ grad, int* status, int n_max, unsigned long long budget_ns, long long n_prep,
-    int chain, int warp_bytes) {
+    int later, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // per warp: the channels' buffers and the candidates of the item
@@ -649,10 +649,10 @@ __global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel
     const LaneTw ltw = lane_twiddles(lane);
     const float Tf = (float)T, inv_fstar = (float)(1.0 / fstar);
     const unsigned long long t0 = budget_ns != 0ULL ? global_ns() : 0ULL;
-    // first items and waits as in loglik_mixed_kernel
-    const int fixed = chain == 0 ? (int)gridDim.x * kWarpsMx : 0;
-    bool waited = chain != 0;
-    if (waited) pdl_launch_dependents();
+    // first items, waits and queues as in loglik_mixed_kernel
+    const bool lead = later >= 0;
+    bool ready = false;   // the preparation's results are visible to this warp
+    if (!lead) pdl_launch_dependents();
     for (;;) {
         // a warp past the time budget takes no further item and flags it
         int item = blockIdx.x * kWarpsMx + warp;
@@ -660,8 +660,10 @@ __global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel
             if (budget_ns != 0ULL && global_ns() - t0 > budget_ns) {
                 atomicOr(status, kStatusBudget);
                 item = n_items;
-            } else if (waited) {
-                item = fixed + atomicAdd(head, 1);
+            } else if (!lead) {
+                item = ready ? atomicAdd(head, 1) : first_item_later(head);
+            } else if (ready) {
+                item = (int)gridDim.x * kWarpsMx - kQueueClosed + atomicAdd(head, 1);
             }
         }
         item = __shfl_sync(0xffffffffu, item, 0);
@@ -673,10 +675,14 @@ __global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel
         const int cnt = (int)(t.c_end - t.c_begin);
         if (lane < cnt) setup_grad_mixed(theta + 8 * (t.c_begin + lane), T, fstar, cands[lane]);
         __syncwarp();
-        if (!waited) {
-            pdl_wait();
-            pdl_launch_dependents();
-            waited = true;
+        if (!ready) {
+            if (lead) {
+                // only after the wait and behind the opened queues may the next part start: its blocks rely on both
+                pdl_wait();
+                if (blockIdx.x == 0 && threadIdx.x == 0) open_queues(head, later);
+                pdl_launch_dependents();
+            }
+            ready = true;
         }
         const WinMeta wm = after_wait(meta)[t.win];
         const Win32* pw = after_wait(prep) + wm.prep_off;
@@ -812,6 +818,7 @@ __global__ void __launch_bounds__(kWarpsMx * 32, GB_GRAD_MINB) grad_mixed_kernel
         __syncwarp();
     }
     pdl_wait();
+    if (lead && blockIdx.x == 0 && threadIdx.x == 0) open_queues(head, later);
 }
 
 }  // namespace

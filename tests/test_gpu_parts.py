@@ -32,3 +32,83 @@ def test_parts_do_not_interact(name, n):
                      th[rows].clone(), prec="mixed")
         for a, b in zip(joint, alone):
             assert torch.isfinite(b).all() and torch.equal(a[rows], b)
+
+
+NAMES = ["loglik_aet", "loglik_phase", "loglik_grad", "loglik_grad_aet"]
+
+
+def _args(name, n, seed):
+    wins, th, data, weights = _problem(seed, SPECS, n)
+    d, w = [_c(x, torch.complex128) for x in data], [_c(x, torch.float64) for x in weights]
+    if not name.endswith("_aet"):
+        d, w = d[:2], w[:2]
+    return wins, d, w, _c(th, torch.float64)
+
+
+@pytest.mark.parametrize("name", ["loglik"] + NAMES)
+@pytest.mark.parametrize("n", [5, 2000])
+def test_parts_read_this_calls_data(name, n):
+    """One layout, other data and weights in each call, eager and replayed:
+    every part must see what the call's own preparation wrote, not the floats
+    that the call before left."""
+    ctx = api.Context(wk.YEAR)
+    sets = [_args(name, n, seed) for seed in (n, n + 1, n + 2)]
+    wins, d, w, th = sets[0]
+    ref = [[x.clone() for x in getattr(api.Context(wk.YEAR), name)(wins, *s[1], *s[2], th, prec="mixed")] for s in sets]
+    assert not torch.equal(ref[0][0], ref[1][0])
+    call = getattr(ctx, name)
+    for k in (0, 1, 2, 1, 0):
+        for a, b in zip(call(wins, *sets[k][1], *sets[k][2], th, prec="mixed"), ref[k]):
+            assert torch.equal(a, b)
+    buf = [x.clone() for x in (*d, *w)]
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        call(wins, *buf, th, prec="mixed")
+        stream.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            out = call(wins, *buf, th, prec="mixed")
+        for k in (0, 1, 2, 1, 0):
+            for x, y in zip(buf, (*sets[k][1], *sets[k][2])):
+                x.copy_(y)
+            graph.replay()
+            for a, b in zip(out, ref[k]):
+                assert torch.equal(a, b)
+    stream.synchronize()
+
+
+@pytest.mark.parametrize("name", ["loglik"] + NAMES)
+def test_time_budget_and_events_over_all_parts(name):
+    """A budget that is not used up, kernel events around the likelihood, and a
+    budget that ends in the middle: the rows that are written are the same bits."""
+    wins, d, w, th = _args(name, 12000, 3)
+    ctx = api.Context(wk.YEAR)
+    call = getattr(ctx, name)
+    ref = [x.clone() for x in call(wins, *d, *w, th, prec="mixed")]
+    ctx.set_time_budget(10.0)
+    for a, b in zip(call(wins, *d, *w, th, prec="mixed"), ref):
+        assert torch.equal(a, b)
+    ctx.check()
+    if "grad" not in name:
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        end.record()
+        ctx.set_kernel_events(start, end)
+        for a, b in zip(call(wins, *d, *w, th, prec="mixed"), ref):
+            assert torch.equal(a, b)
+        torch.cuda.synchronize()
+        assert start.elapsed_time(end) > 0.0
+    for budget in (5e-9, 10e-6, 200e-6):   # the first: warps may end before they take an item
+        ctx.set_time_budget(budget)
+        got = call(wins, *d, *w, th, prec="mixed")
+        try:
+            ctx.check()
+            full = True
+        except api.GBError:
+            full = False
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b) if full else ((a == b) | (a == 0.0)).all()
+    ctx.set_time_budget(0.0)
+    for a, b in zip(call(wins, *d, *w, th, prec="mixed"), ref):
+        assert torch.equal(a, b)
+    ctx.check()
