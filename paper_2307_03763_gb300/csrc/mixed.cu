@@ -115,7 +115,8 @@ int launch_loglik_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const d
         int grid = sms * bpsm;
         const int need = (n_items + kWarpsMx - 1) / kWarpsMx;
         if (grid > need) grid = need;
-        const bool dependent = chain == 0 ? !ev_start : held <= kHeldMax;
+        // under a time budget each kernel has the GPU to itself, as its clock assumes
+        const bool dependent = ctx->budget_ns == 0ULL && (chain == 0 ? !ev_start : held <= kHeldMax);
         e = launch_mixed_part(kfn, grid, smem, s, plan.d_win, plan.d_meta, plan.d_prep, plan.d_tiles + first, n_items,
                               plan.d_head + part, tabset32(ctx), (const float2*)ctx->d_tw32, ctx->obs.T_obs,
                               transfer_frequency(ctx), theta, logL, dh, hh, dh_im, ctx->d_status, nmax,

@@ -45,7 +45,8 @@ int launch_grad_mixed(gb_ctx* ctx, const Plan& plan, const double* dA, const dou
         void* args[] = {(void*)&plan.d_win, (void*)&plan.d_meta, (void*)&plan.d_prep, (void*)&items, &n_it, &head,
                         &tabs, &tw, &Tobs, &fstar, (void*)&theta, &logL, &grad, &status, &n_mx, &budget, &n_prep,
                         &later, &warp_bytes};
-        e = launch_chained(kfn, grid, smem, s, args, chain == 0 || held <= kHeldMax);
+        // under a time budget each kernel has the GPU to itself, as its clock assumes
+        e = launch_chained(kfn, grid, smem, s, args, budget == 0ULL && (chain == 0 || held <= kHeldMax));
         held = smem * bpsm;
         ++chain;
         ++ctx->launches;

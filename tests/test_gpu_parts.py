@@ -2,6 +2,7 @@
 a candidate's results do not depend on what else the call holds, so every
 window must get the same bits alone as beside windows of the other parts.
 Candidate counts give items of one, an odd number and the most candidates."""
+import numpy as np
 import pytest
 import torch
 
@@ -110,5 +111,40 @@ def test_time_budget_and_events_over_all_parts(name):
             assert torch.equal(a, b) if full else ((a == b) | (a == 0.0)).all()
     ctx.set_time_budget(0.0)
     for a, b in zip(call(wins, *d, *w, th, prec="mixed"), ref):
+        assert torch.equal(a, b)
+    ctx.check()
+
+
+@pytest.mark.parametrize("grad", [False, True])
+def test_time_budget_leaves_the_preparation_out(grad):
+    """A window of four million bins takes the preparation many times as long
+    as the kernel takes for its candidates: a budget between the two suffices."""
+    n = 200000
+    src = wk.source(2e-3, 1e-17, 1e-22, np.random.default_rng(1))
+    th = torch.as_tensor(wk.uniform_box(src, np.array([1e-8, 1e-17, 0.1, 0.1, 1e-23, 0.1, 0.1, 0.1]), n,
+                                        np.random.default_rng(2)), device="cuda")
+    ctx = api.Context(wk.YEAR)
+
+    def problem(W):
+        win = [(int(2e-3 * wk.YEAR) - 64, W, 128, 0, 0, n)]
+        d, w = torch.zeros(W, dtype=torch.complex128, device="cuda"), torch.ones(W, dtype=torch.float64, device="cuda")
+        call = ctx.loglik_grad if grad else ctx.loglik
+        return lambda: call(win, d, d, w, w, th, prec="mixed")
+
+    def seconds(f):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        f()
+        a.record()
+        out = f()
+        b.record()
+        torch.cuda.synchronize()
+        return a.elapsed_time(b) * 1e-3, [x.clone() for x in out]
+
+    kernel, _ = seconds(problem(128))
+    long = problem(1 << 22)
+    total, ref = seconds(long)
+    assert total > 8 * kernel
+    ctx.set_time_budget(total / 4)
+    for a, b in zip(long(), ref):
         assert torch.equal(a, b)
     ctx.check()
