@@ -27,8 +27,8 @@
 // theta_m, its difference Delta gives dp = Sh sin a Delta/2, dq = Dh cos a
 // Delta/2 to first order.
 //
-// Everything here also compiles for the host, where the tests of the index
-// arithmetic and of the rounding run.
+// Everything here also compiles for the host, where tests/test_fx64_host.py
+// checks the rounding against long double and that no sum wraps.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -217,7 +217,7 @@ struct MidFx {
     fx nu[3], nv[3];           // n.u, n.v, Q62
     fx K;                      // K / 512 s, Q60
     uint64_t ph;               // carrier phase, 2^-64 cycles
-    int ep[3];                 // eps of the receivers, Q57
+    int ep[3];                 // eps of the receivers, Q56
     fx co[3], si[3];           // exp(i theta) of the arms, Q62
     Bx C1, S1;                 // amplitude polynomials, Q62
 };
@@ -263,7 +263,7 @@ GB_FX void middle_fx(const CandFx& c, const GeoFx& g, int krho_q30, int n, int l
         ph -= (uint64_t)mul(bal(t), Kb).get<8>();
     }
     m.ph = ph;
-    // eps of the three receivers in Q57 (see the head of the file); k.rho_j in
+    // eps of the three receivers in Q56 (see the head of the file); k.rho_j in
     // units of (L/c)/3 s: the differences of the arms' k.n
     int ep0, ep1, ep2;
     {
@@ -272,27 +272,27 @@ GB_FX void middle_fx(const CandFx& c, const GeoFx& g, int krho_q30, int n, int l
         const int s0 = Kh + (int)(wide(kr0, krho_q30) >> 30), s1 = Kh + (int)(wide(kr1, krho_q30) >> 30),
                   s2 = Kh + (int)(wide(kr2, krho_q30) >> 30);   // (2K + k.rho)/1024 s, Q29
         const int t0 = (int)(wide(kr0, s0) >> 29), t1 = (int)(wide(kr1, s1) >> 29), t2 = (int)(wide(kr2, s2) >> 29);
-        ep0 = (int)(wide(t0, c.FD) >> 30);   // Q29 + Q58 - 30 = Q57
-        ep1 = (int)(wide(t1, c.FD) >> 30);
-        ep2 = (int)(wide(t2, c.FD) >> 30);
+        ep0 = (int)(wide(t0, c.FD) >> 31);   // Q29 + Q58 - 31 = Q56
+        ep1 = (int)(wide(t1, c.FD) >> 31);
+        ep2 = (int)(wide(t2, c.FD) >> 31);
     }
     m.ep[0] = ep0;
     m.ep[1] = ep1;
     m.ep[2] = ep2;
     // arm phase factors; z = 3 theta + 3 (eps_i + eps_j)/2
     fx c0, s0, c1, s1, c2, s2;
-    cis_third<TIER>(b[1] - b[2] + 48ll * (ep0 + ep1), c0, s0);   // Q57 -> Q62 and 3/2: x 48
-    cis_third<TIER>(b[2] - b[0] + 48ll * (ep1 + ep2), c1, s1);
+    cis_third<TIER>(b[1] - b[2] + 96ll * (ep0 + ep1), c0, s0);   // Q56 -> Q62 and 3/2: x 96
+    cis_third<TIER>(b[2] - b[0] + 96ll * (ep1 + ep2), c1, s1);
     {
         const Bx c0b = bal(c0), s0b = bal(s0), c1b = bal(c1), s1b = bal(s1);
         Dot dc = mul(c0b, c1b), ds = mul(s0b, c1b);
         dc.add(bal(-s0), s1b);
         ds.add(c0b, s1b);
         // conjugate of the product, turned by the sum of the three mean eps
-        const int sg = ep0 + ep1 + ep2;   // Q57
+        const int sg = ep0 + ep1 + ep2;   // Q56
         c2 = dc.get<2>();
         s2 = -ds.get<2>();
-        const fx cr = wide((int)(s2 >> 32), sg) >> 25, sr = wide((int)(c2 >> 32), sg) >> 25;   // Q30 + Q57 -> Q62
+        const fx cr = wide((int)(s2 >> 32), sg) >> 24, sr = wide((int)(c2 >> 32), sg) >> 24;   // Q30 + Q56 -> Q62
         c2 -= cr;
         s2 += sr;
     }
@@ -381,9 +381,9 @@ GB_FX void sample_fx(const CandFx& c, const GeoFx& g, const FxTw* tw, int krho_q
         const Bx Sh = bal(sp + sm), Dh = bal(sp - sm);
         const fx p = mul(Sh, C1).get(), q = mul(Dh, S1).get();
         // dp = Sh S1 Delta/2, dq = Dh C1 Delta/2 in Q58, Delta = eps of the + receiver - eps of the - one
-        const int dl = m.ep[k == 2 ? 0 : k + 1] - m.ep[k];   // Q57
+        const int dl = m.ep[k == 2 ? 0 : k + 1] - m.ep[k];   // Q56
         const int ss = (int)(wide(Sh.h, S1.h) >> 30), dc = (int)(wide(Dh.h, C1.h) >> 30);   // Q30
-        const fx dp = (wide(ss, dl) >> 30) * 4, dq = (wide(dc, dl) >> 30) * 4;   // Q57 of value/2 = Q58; x 4: Q60
+        const fx dp = (wide(ss, dl) >> 29) * 4, dq = (wide(dc, dl) >> 29) * 4;   // Q57 of value/2 = Q58; x 4: Q60
         // A sqrt2 = Z - X, E sqrt6 = X - 2Y + Z, T sqrt3 = X + Y + Z: coefficients of H_k
         fx ar, ai, er, ei;
         if (k == 0) {
@@ -512,9 +512,12 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     const double fdT = fd * T, fdT_e = fma(fd, T, -fdT), c2h = 0.5 * (fdT * T),
                  c2l = 0.5 * (fma(fdT, T, -(fdT * T)) + fdT_e * T), c2r = rint(c2h);
     const double FD = pi * fd * (arm_c / 3.0) * 1024.0, w1 = 512.0 * fd * T, w2 = 131072.0 * fd;
-    // arm_c: k.rho/1024 s must stay small against K/512 s (the eps terms are 32-bit)
+    // The eps terms are 32-bit: with k.rho of up to sqrt3 (L/3c), |K| <= 500 s
+    // and arm_c < 300 s, |k.rho (2K + k.rho)| stays below 1.99 units, so |eps|
+    // below 1.99 2^29 (Q56) for FD 2^58 < 2^31 (rounded: hence not up to
+    // 2^-27), and the difference of two below 3.3 2^29.
     const bool ok = f0 > 0.0 && xmax <= 1.3 && fabs(eta) <= 0x1p-10 && fabs(Fc) < 31.0 && fabs(Fs) < 31.0 &&
-                    fabs(c2h) < 0x1p30 && fabs(FD) < 0x1p-27 && fabs(w1) < 0.9 && fabs(w2) < 0.2 && arm_c < 300.0 &&
+                    fabs(c2h) < 0x1p30 && fabs(FD) < 0x1.fffffp-28 && fabs(w1) < 0.9 && fabs(w2) < 0.2 && arm_c < 300.0 &&
                     fabs(delta) < 0x1p40 && fabs(phi0) < 0x1p30;
     c.tier = !ok ? -1 : xmax <= 0.5 ? 0 : 1;
     if (!ok) return;

@@ -157,9 +157,9 @@ GB_FX void adjoint_fx(const CandFx& c, const CandGFx& cg, const GeoFx& g, const 
         const fx Sg_ = dpl + dm, Dd_ = dpl - dm;
         const Bx Sg = bal(Sg_), Dd = bal(Dd_), kn = bal(m.kn[k]);
         const fx p = mul(Sh, m.C1).get(), q = mul(Dh, m.S1).get();   // Q60
-        const int dl = m.ep[k == 2 ? 0 : k + 1] - m.ep[k];           // Q57
+        const int dl = m.ep[k == 2 ? 0 : k + 1] - m.ep[k];           // Q56
         const int ss = (int)(wide(Sh.h, m.S1.h) >> 30), dc = (int)(wide(Dh.h, m.C1.h) >> 30);
-        const fx dp = (wide(ss, dl) >> 30) * 4, dq = (wide(dc, dl) >> 30) * 4;   // Q60
+        const fx dp = (wide(ss, dl) >> 29) * 4, dq = (wide(dc, dl) >> 29) * 4;   // Q60
         // nu = (p - i dq) P + (dp + i q) R: Q60
         const Bx pb = bal(p), qb = bal(q), dpb = bal(dp), dqb = bal(dq);
         Dot x = mul(pb, Prb), y = mul(pb, Pib);
@@ -207,7 +207,7 @@ GB_FX void adjoint_fx(const CandFx& c, const CandGFx& cg, const GeoFx& g, const 
         const float gR = ((float)Gr.h * (float)Rrb.h - (float)Gi.h * (float)Rib.h) * 0x1p-56f;
         const float gP = ((float)Gr.h * (float)Pib.h + (float)Gi.h * (float)Prb.h) * 0x1p-56f;
         pk[k] = 0.5f * (gR * S * s1 + gP * D * c1);
-        xk[k] = 0.5f * ((float)dl * 0x1p-57f) * hi_f(m.a, 0x1p-30f) *
+        xk[k] = 0.5f * ((float)dl * 0x1p-56f) * hi_f(m.a, 0x1p-30f) *
                 (gR * hi_f(Dd_, 0x1p-30f) * s1 + gP * hi_f(Sg_, 0x1p-30f) * c1);
     }
     // theta_k = (b_p - b_q)/3: its share of a0 d/da and of d/d(k.n)

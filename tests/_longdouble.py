@@ -9,12 +9,14 @@ PI = L("3.14159265358979323846264338327950288")
 C, AU, ARM, YEAR = L(299792458), L(1.495978707e11), L(2.5e9), L(31557600)
 
 
-def template_aet(theta, N, T):
-    """q (int64) and the A, E, T templates on bins q - N/2 ... q + N/2 - 1, clongdouble."""
+def template_aet(theta, N, T, step=None):
+    """q (int64) and the A, E, T templates on bins q - N/2 ... q + N/2 - 1, clongdouble.
+    step (8 long doubles): the parameters' offset from theta, whose carrier bin and delta's rounding are kept."""
     th = np.asarray(theta, dtype=np.float64)
     f0T = th[:, 0] * float(T)
     q = np.floor((f0T + ((0.5 * th[:, 1]) * float(T)) * float(T)) + 0.5)
-    delta = (f0T - q).astype(L)[:, None]
+    step = np.zeros(8, L) if step is None else step
+    delta = (f0T - q).astype(L)[:, None] + step[0] * L(T)
     T = L(T)
     n = np.arange(N).astype(L)
     t = n * T / L(N)
@@ -25,7 +27,7 @@ def template_aet(theta, N, T):
         b = 2 * PI * i / 3
         x.append((AU * np.cos(a) + AU * ecc / 2 * (np.cos(2 * a - b) - 3 * np.cos(b)),
                   AU * np.sin(a) + AU * ecc / 2 * (np.sin(2 * a - b) - 3 * np.sin(b)), -s3 * AU * ecc * np.cos(a - b)))
-    f0, fd, be, la, A, io, ps, ph = (th[:, j].astype(L)[:, None] for j in range(8))
+    f0, fd, be, la, A, io, ps, ph = (th[:, j].astype(L)[:, None] + step[j] for j in range(8))
     sb, cb, sl, cl = np.sin(be), np.cos(be), np.sin(la), np.cos(la)
     k, u, v = (-cb * cl, -cb * sl, -sb), (sb * cl, sb * sl, -cb), (sl, -cl)
     c2, s2, ci = np.cos(2 * ps), np.sin(2 * ps), np.cos(io)

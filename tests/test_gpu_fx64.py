@@ -132,3 +132,24 @@ def test_gradient_of_non_finite_data_is_nan():
     bad[N // 2] = float("nan")
     _, g = api.Context(T).loglik_grad(win, bad, d, w, w, torch.as_tensor(th, device="cuda"))
     assert torch.isnan(g).all()
+
+
+# the eps terms' coefficient pi fdot (L/c)/3 1024 is admitted up to 2^-27
+FDOT_MAX = 2.0 ** -27 / (math.pi * 2.5e9 / 299792458.0 / 3.0 * 1024.0)
+
+
+@pytest.mark.parametrize("f0", [16e-3, 20e-3, 24e-3])
+@pytest.mark.parametrize("frac", [0.93, 0.999, 1.001, -0.93, -0.999])
+def test_templates_at_the_chirp_limit(f0, frac):
+    """Sky positions around those where the differences of the receivers' chirp terms are largest."""
+    T, N, n = 0.5 * wk.YEAR, 1024, 60
+    th = candidates(f0, frac * FDOT_MAX, n, int(1e4 * f0))
+    rng = np.random.default_rng(n)
+    th[2:, 2] = rng.uniform(-0.5, 0.5, n - 2)
+    th[2:, 3] = np.where(np.arange(n - 2) % 2, 0.70, 3.84) + rng.uniform(-0.6, 0.6, n - 2)
+    out = api.Context(T).waveform_aet(torch.as_tensor(th, device="cuda"), N)
+    q, ref = ld.template_aet(th, N, T)
+    assert np.array_equal(out[3].cpu().numpy(), q)
+    norm = lambda x: np.sqrt((np.abs(x) ** 2).sum(1).astype(np.float64))  # noqa: E731
+    for h, r in zip(out[:2], ref[:2]):
+        assert np.all(norm(h.cpu().numpy() - r) <= tolerance(th, T) * norm(r))
