@@ -252,8 +252,8 @@ class Context:
         """The layout of a window list, kept by value: a list whose rows equal a
         kept one's (tuples of ints; 70 us for 2,048 windows) is not converted
         again (0.8 ms)."""
+        key = windows = tuple(windows)   # once: an iterator is spent after it
         try:
-            key = tuple(windows)
             lay = self._layouts.get(key)
         except TypeError:   # rows that cannot be hashed (lists, arrays)
             key = lay = None

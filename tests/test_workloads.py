@@ -121,3 +121,18 @@ def test_layouts_are_kept_by_value():
     assert ctx._layout([(5, 32, 32, 0, 0, 3), (9, 32, 64, 32, 4, 4)]).covered == -1
     assert ctx._layout([(5, 32, 32, 0, 0, 3), (9, 32, 64, 32, 2, 4)]).covered == -1
     assert ctx._layout([]).covered == 0
+
+
+@pytest.mark.parametrize("n", [2, 70])
+def test_layouts_of_iterators(n):
+    """Windows that can be walked only once, with hashable rows and others, give the list's layout."""
+    from paper_2307_03763_gb300 import api
+    rows = [(5 + i, 32, 32, 32 * i, 3 * i, 3) for i in range(n)]
+    arr = np.array(rows)
+    for make in (lambda: iter(rows), lambda: (list(r) for r in rows), lambda: zip(*arr.T), lambda: map(tuple, arr),
+                 lambda: iter(arr), lambda: (tuple(float(x) for x in r) for r in rows), lambda: map(iter, rows)):
+        ctx = api.Context.__new__(api.Context)
+        ctx._layouts = {}
+        lay = ctx._layout(make())
+        assert (lay.n, lay.covered, lay.kmax) == (n, 3 * n, 3) and bytes(lay.arr) == bytes(api.windows_array(rows))
+        assert ctx._layout(make()) is lay and ctx._layout(rows) is lay
