@@ -32,11 +32,14 @@
 #pragma once
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #ifdef __CUDACC__
 #define GB_FX __host__ __device__ __forceinline__
+#define GB_FXN __host__ __device__
 #else
 #define GB_FX inline
+#define GB_FXN
 #endif
 
 namespace gb {
@@ -580,6 +583,112 @@ GB_FX void setup_fx(const double* th, double T, double arm_c, double delta, int 
     c.sA = amp * 0.70710678118654752;
     c.sE = amp * 0.40824829046386302;
     c.sT = amp * 0.57735026918962576 * ldexp(1.0, -c.tsh);
+}
+
+// Index of element e in a transform buffer: the low three bits XORed with the
+// higher groups of three, so that eight lanes whose indices differ in any
+// three neighbouring bits (every stage of the transform, the bit-reversed
+// stores and the reads in order) meet eight different 16-byte bank groups.
+GB_FX int sw(int e) { return e ^ ((e >> 3) & 7) ^ ((e >> 6) & 7) ^ ((e >> 9) & 1); }
+
+// synchronisation of the NT threads that share a transform (one thread: none)
+template <int NT>
+GB_FX void sync_nt() {
+#ifdef __CUDA_ARCH__
+    if (NT == 32) __syncwarp();
+    else __syncthreads();
+#endif
+}
+
+GB_FX fx double_bits(double v) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(v);
+#else
+    fx b;
+    memcpy(&b, &v, sizeof b);
+    return b;
+#endif
+}
+
+// a fixed-point complex value, or, after the last stage, the bits of two doubles
+struct alignas(16) Z64 {
+    fx x, y;
+};
+GB_FX Z64 zadd(Z64 a, Z64 b) { return {a.x + b.x, a.y + b.y}; }
+GB_FX Z64 zsub(Z64 a, Z64 b) { return {a.x - b.x, a.y - b.y}; }
+GB_FX Z64 zmi(Z64 a) { return {a.y, -a.x}; }   // times -i
+GB_FX Z64 zmul(Z64 a, const FxTw& w) {   // times co - i si
+    const Bx r = bal(a.x), i = bal(a.y), mr = bal(-a.x);
+    Dot re = mul(r, w.co), im = mul(mr, w.si);
+    re.add(i, w.si);
+    im.add(i, w.co);
+    return {re.get<2>(), im.get<2>()};
+}
+GB_FX Z64 zout(Z64 a, double s, bool last) {
+    if (!last) return a;
+    return {double_bits((double)a.x * s), double_bits((double)a.y * s)};
+}
+
+// In-place FFT of nch buffers (stride elements apart): bit-reversed input,
+// natural order output, as doubles times sc[ch] or (RAW) as it is.  Radix-2 decimation in time,
+// two stages at a time (three twiddle products per four elements; the first
+// two stages have none), the odd stage last.  Bound by the integer products
+// of the twiddles.
+template <int NT, bool RAW = false>
+GB_FXN void fft_fx(Z64* buf, int stride, int nch, int lg, const FxTw* tw, const double* sc, int lane) {
+    const int N = 1 << lg;
+    for (int q = lane; q < N / 4; q += NT) {
+        const int i0 = sw(4 * q), i1 = sw(4 * q + 1), i2 = sw(4 * q + 2), i3 = sw(4 * q + 3);
+        for (int ch = 0; ch < nch; ++ch) {
+            Z64* p = buf + (size_t)ch * stride;
+            const Z64 x0 = p[i0], x1 = p[i1], x2 = p[i2], x3 = p[i3];
+            const Z64 a = zadd(x0, x1), b = zsub(x0, x1), c = zadd(x2, x3), d = zmi(zsub(x2, x3));
+            p[i0] = zadd(a, c);
+            p[i1] = zadd(b, d);
+            p[i2] = zsub(a, c);
+            p[i3] = zsub(b, d);
+        }
+    }
+    sync_nt<NT>();
+    int s = 2;
+    for (; s + 2 <= lg; s += 2) {
+        const bool last = !RAW && s + 2 == lg;
+        const int h = 1 << s;
+        for (int q = lane; q < N / 4; q += NT) {
+            const int j = q & (h - 1), e = ((q >> s) << (s + 2)) + j;
+            const int i0 = sw(e), i1 = sw(e + h), i2 = sw(e + 2 * h), i3 = sw(e + 3 * h);
+            // exp(-2 pi i m j / 4h), m = 2, 1, 3; entry k >= 512 is minus entry k - 512
+            const FxTw w1 = tw[j << (9 - s)], w2 = tw[j << (8 - s)];
+            const int k3 = (3 * j) << (8 - s);
+            const FxTw w3 = tw[k3 & 511];
+            for (int ch = 0; ch < nch; ++ch) {
+                Z64* p = buf + (size_t)ch * stride;
+                const Z64 x0 = p[i0], x1 = zmul(p[i1], w1), x2 = zmul(p[i2], w2);
+                Z64 x3 = zmul(p[i3], w3);
+                if (k3 & 512) x3 = {-x3.x, -x3.y};
+                const Z64 a = zadd(x0, x1), b = zsub(x0, x1), c = zadd(x2, x3), d = zmi(zsub(x2, x3));
+                p[i0] = zout(zadd(a, c), sc[ch], last);
+                p[i1] = zout(zadd(b, d), sc[ch], last);
+                p[i2] = zout(zsub(a, c), sc[ch], last);
+                p[i3] = zout(zsub(b, d), sc[ch], last);
+            }
+        }
+        sync_nt<NT>();
+    }
+    if (s < lg) {
+        const int h = 1 << s;
+        for (int q = lane; q < N / 2; q += NT) {
+            const int i0 = sw(q), i1 = sw(q + h);
+            const FxTw w = tw[q << (9 - s)];
+            for (int ch = 0; ch < nch; ++ch) {
+                Z64* p = buf + (size_t)ch * stride;
+                const Z64 a = p[i0], b = zmul(p[i1], w);
+                p[i0] = zout(zadd(a, b), sc[ch], !RAW);
+                p[i1] = zout(zsub(a, b), sc[ch], !RAW);
+            }
+        }
+        sync_nt<NT>();
+    }
 }
 
 }  // namespace gb

@@ -43,6 +43,29 @@ GB_FX fx sinc_dy(Bx y) {
     return step64<2>(r, y, -768614336404564650ll);
 }
 
+// Scale 2^k that takes a residual to integers for its transform.  The sum of
+// |re| + |im| over the bins (of the channel where it is largest) bounds the
+// transform and everything on the way to it, and is brought below 2^62; the
+// largest component times N would leave log2 N bits unused where one bin
+// dominates.  The sum is taken from the components' high words, in units of
+// 2^-19 of the largest component's power of two, each rounded up (FP64 sums:
+// 2% of the gradient's time).  hi, top: high words of |component| and of the
+// largest one; at most 2 x 1024 shares of 2^20 + 1 are added.
+GB_FX unsigned residual_share(unsigned hi, unsigned top) {
+    const unsigned d = (top >> 20) - (hi >> 20);
+    return (((hi & 0xFFFFFu) | 0x100000u) >> (d < 30u ? d + 1u : 31u)) + 1u;
+}
+GB_FX int residual_shift(unsigned sum, unsigned top) {
+    int b = 0;   // sum < 2^b
+#ifdef __CUDA_ARCH__
+    b = 32 - __clz((int)sum);
+#else
+    while (b < 32 && sum >> b) ++b;
+#endif
+    const int k = 62 - (b - 19 + (int)(top >> 20) - 1023);
+    return k < 1000 ? k : 1000;
+}
+
 struct CandGFx {
     Bx a0, a3;                   // Q62, a0 and a0/3
     Bx eta;                      // Q70, fdot T/f0

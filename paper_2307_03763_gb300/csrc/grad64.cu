@@ -15,9 +15,13 @@
 // Measured on GB300, 64 windows x 512 candidates at N = 256: 33.8 ms with every
 // step in double (FP64 pipe 84% busy), 4.8 ms in this form (8,900 warp
 // instructions per 32 samples, the multiply pipe 54-65% and the FP64 pipe 35%
-// busy with eight warps per SM, the most that 255 registers leave).  Error of the
-// gradients against 113-bit arithmetic: 1e-15 ... 8e-15 of their norm per
-// parameter, where the double form had 3e-15 ... 5e-14.
+// busy with eight warps per SM, the most that 255 registers leave).  Error of a
+// gradient against 113-bit arithmetic, largest parameter over the norm, for
+// data of a source and noise | of one loud bin: median 3e-16 | 3e-16 ... 1.6e-15,
+// where the double form had 6e-16 ... 5e-15 | 1.3e-15 ... 8e-15 (0.4-23 mHz,
+// N = 32-1024); beside a source, where the gradient all but vanishes, 2e-14
+// against 3e-14.  The adjoint transform alone, N = 1024: 2e-16 (white residual)
+// and 2e-17 (one loud bin) of its norm, in double 4e-16.
 //
 // Candidates outside the fixed-point ranges take the plain double form: each
 // sample's forward values (the fast/slow response of
@@ -539,9 +543,20 @@ __device__ __noinline__ void sweep_fx(const CandGT& c, const Geo& g, const FxTab
     }
     top = __reduce_max_sync(0xffffffffu, top);
     __syncwarp();
-    // to integers below 2^(61 - lg), A's normalisation for every channel, and
-    // into bit-reversed order
-    const int k = min(1000, 61 - lg - ((int)(top >> 20) - 1022));
+    // to integers, A's normalisation for every channel, and into bit-reversed order
+    unsigned share[NCH] = {};
+    for (int i = lane; i < N; i += 32) {
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            const C r = buf[ch * stride + i];
+            share[ch] += residual_share(abs_hi(r.x), top) + residual_share(abs_hi(r.y), top);
+        }
+    }
+    unsigned sum = 0;
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch) sum = max(sum, __reduce_add_sync(0xffffffffu, share[ch]));
+    __syncwarp();   // every bin is read before it is overwritten
+    const int k = residual_shift(sum, top);
     const double s0 = scalbn(1.0, k);
     const double sc[3] = {s0, s0 * 0.57735026918962576, s0 * 0.81649658092772603};
     Z64* z = (Z64*)buf;

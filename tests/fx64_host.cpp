@@ -116,4 +116,30 @@ void host_gradients(int B, const double* theta, const double* delta, double T, d
         finish_gfx(fin, T, sums, 0x1p-60 * 0x1p60, grad + 8 * b);
     }
 }
+
+// transform of B residuals (N complex each): N integers and the power of two that they carry
+void host_transform(int B, int lg, const double* r, fx* out, int* power) {
+    const auto tw = twiddles();
+    const int N = 1 << lg;
+    const double one[3] = {1.0, 1.0, 1.0};
+    std::vector<Z64> z(N);
+    for (int b = 0; b < B; ++b) {
+        const double* x = r + (size_t)b * 2 * N;
+        auto high = [&](int i) { return (unsigned)((uint64_t)double_bits(fabs(x[i])) >> 32); };
+        unsigned top = 0, sum = 0;
+        for (int i = 0; i < 2 * N; ++i) top = high(i) > top ? high(i) : top;
+        for (int i = 0; i < 2 * N; ++i) sum += residual_share(high(i), top);
+        const int k = power[b] = residual_shift(sum, top);
+        for (int i = 0; i < N; ++i) {
+            int j = 0;
+            for (int q = 0; q < lg; ++q) j |= ((i >> q) & 1) << (lg - 1 - q);
+            z[sw(j)] = Z64{to_fx(ldexp(x[2 * i], k), 1.0), to_fx(ldexp(x[2 * i + 1], k), 1.0)};
+        }
+        fft_fx<1, true>(z.data(), N, 1, lg, tw.data(), one, 0);
+        for (int i = 0; i < N; ++i) {
+            out[((size_t)b * N + i) * 2] = z[sw(i)].x;
+            out[((size_t)b * N + i) * 2 + 1] = z[sw(i)].y;
+        }
+    }
+}
 }
