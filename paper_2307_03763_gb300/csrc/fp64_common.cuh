@@ -168,7 +168,7 @@ __device__ void setup64(const double* th, double T, double inv_fstar, double del
     // link-transfer series: first omitted term below 1e-17 for the largest
     // argument X = f (1 + |k.n|)/(2 f*) <= f_max / f*
     const double xmax = fmax(fabs(f0), fabs(f0 + fd * T)) * inv_fstar;
-    c.J = xmax <= 2.35 ? 16 : 0;
+    c.J = xmax <= 0.22 ? 6 : xmax <= 0.5 ? 8 : xmax <= 1.3 ? 12 : xmax <= 2.35 ? 16 : 0;
     double sD, cD;
     sincos(f0 * inv_fstar, &sD, &cD);
     c.D0r = cD;
@@ -185,10 +185,13 @@ __device__ __forceinline__ C64 nHn(const Cand64& c, double nx, double ny, double
 }
 
 // sinc(X) exp(-iX): J+1 terms of the series of (1 - e^{-2iX})/(2iX) split into
-// real and imaginary parts (Horner in y = -4X^2); J = 0: direct evaluation
-template <int J>
-__device__ __forceinline__ C64 transfer64(double X) {
-    if constexpr (J == 0) {
+// real and imaginary parts (Horner in y = -4X^2), or evaluated directly.  J is
+// a run-time number: one length for all (16) took 20% longer at 4 mHz (160,000
+// likelihoods of drifting candidates, N = 256: 49.8 -> 41.1 ms), an unrolled
+// copy per length takes registers from the kernels' fixed-point form.
+template <bool SERIES>
+__device__ __forceinline__ C64 transfer64(double X, int J) {
+    if constexpr (!SERIES) {
         double sX, cX;
         sincos(X, &sX, &cX);
         const double sinc = (X != 0.0) ? sX / X : 1.0;
@@ -196,7 +199,7 @@ __device__ __forceinline__ C64 transfer64(double X) {
     } else {
         const double y = -4.0 * X * X;
         double re = kInvFact64[2 * J + 1], im = kInvFact64[2 * J + 2];
-#pragma unroll
+#pragma unroll 2
         for (int j = J - 1; j >= 0; --j) {
             re = fma(re, y, kInvFact64[2 * j + 1]);
             im = fma(im, y, kInvFact64[2 * j + 2]);
@@ -206,9 +209,9 @@ __device__ __forceinline__ C64 transfer64(double X) {
 }
 
 // -i a sinc(X) exp(-iX) G exp(i Psi)
-template <int J>
-__device__ __forceinline__ C64 link64(double a, double X, C64 G, C64 rx) {
-    const C64 t = transfer64<J>(X);
+template <bool SERIES>
+__device__ __forceinline__ C64 link64(double a, double X, C64 G, C64 rx, int J) {
+    const C64 t = transfer64<SERIES>(X, J);
     const C64 tr = {a * t.x, a * t.y};
     const C64 z = cmul(cmul(tr, G), rx);
     return {z.y, -z.x};                                    // times -i
@@ -223,7 +226,7 @@ __device__ __forceinline__ C64 link64(double a, double X, C64 G, C64 rx) {
 // the whole CTA, `lane` the thread index); each sample and each butterfly is
 // computed by the same code whichever thread takes it, so the bits do not
 // depend on NT (here and in the fixed-point form).
-template <int J, int NT>
+template <bool SERIES, int NT>
 __device__ __noinline__ void template64(const Cand64& c, const Geo64& g, const OrbitTables64& tab, const C64* tw,
                            C64* bufA, C64* bufE, C64* bufT, int lane) {
     const int N = g.N;
@@ -250,22 +253,22 @@ __device__ __noinline__ void template64(const Cand64& c, const Geo64& g, const O
             const double nx = tab.arm[0 * N + n], ny = tab.arm[1 * N + n], nz = tab.arm[2 * N + n];
             const double kn = c.k[0] * nx + c.k[1] * ny + c.k[2] * nz;
             const C64 G = nHn(c, nx, ny, nz);
-            z01 = link64<J>(a, a * (1.0 - kn), G, rx[1]);
-            z10 = link64<J>(a, a * (1.0 + kn), G, rx[0]);
+            z01 = link64<SERIES>(a, a * (1.0 - kn), G, rx[1], c.J);
+            z10 = link64<SERIES>(a, a * (1.0 + kn), G, rx[0], c.J);
         }
         {
             const double nx = tab.arm[3 * N + n], ny = tab.arm[4 * N + n], nz = tab.arm[5 * N + n];
             const double kn = c.k[0] * nx + c.k[1] * ny + c.k[2] * nz;
             const C64 G = nHn(c, nx, ny, nz);
-            z12 = link64<J>(a, a * (1.0 - kn), G, rx[2]);
-            z21 = link64<J>(a, a * (1.0 + kn), G, rx[1]);
+            z12 = link64<SERIES>(a, a * (1.0 - kn), G, rx[2], c.J);
+            z21 = link64<SERIES>(a, a * (1.0 + kn), G, rx[1], c.J);
         }
         {
             const double nx = tab.arm[6 * N + n], ny = tab.arm[7 * N + n], nz = tab.arm[8 * N + n];
             const double kn = c.k[0] * nx + c.k[1] * ny + c.k[2] * nz;
             const C64 G = nHn(c, nx, ny, nz);
-            z20 = link64<J>(a, a * (1.0 - kn), G, rx[0]);
-            z02 = link64<J>(a, a * (1.0 + kn), G, rx[2]);
+            z20 = link64<SERIES>(a, a * (1.0 - kn), G, rx[0], c.J);
+            z02 = link64<SERIES>(a, a * (1.0 + kn), G, rx[2], c.J);
         }
         // D = exp(-i f/f*) = exp(-i f0/f*) exp(-i th), th = fdot t / f*: a short
         // series while |th| <= 1/64 (terms to th^7, first omitted below 1e-19)
@@ -326,8 +329,8 @@ __device__ __noinline__ void template64(const Cand64& c, const Geo64& g, const O
 template <int NT>
 __device__ void template_plain(const CandT& c, const Geo64& g, const OrbitTables64& tab, const C64* tw, C64* bufA,
                                C64* bufE, C64* bufT, int lane) {
-    if (c.d.J == 16) template64<16, NT>(c.d, g, tab, tw, bufA, bufE, bufT, lane);
-    else template64<0, NT>(c.d, g, tab, tw, bufA, bufE, bufT, lane);
+    if (c.d.J) template64<true, NT>(c.d, g, tab, tw, bufA, bufE, bufT, lane);
+    else template64<false, NT>(c.d, g, tab, tw, bufA, bufE, bufT, lane);
     for (int i = lane; i < g.N; i += NT) {
         bufA[i] = cscale(bufA[i], g.scale);
         bufE[i] = cscale(bufE[i], g.scale);

@@ -153,3 +153,19 @@ def test_templates_at_the_chirp_limit(f0, frac):
     norm = lambda x: np.sqrt((np.abs(x) ** 2).sum(1).astype(np.float64))  # noqa: E731
     for h, r in zip(out[:2], ref[:2]):
         assert np.all(norm(h.cpu().numpy() - r) <= tolerance(th, T) * norm(r))
+
+
+@pytest.mark.parametrize("x", [0.05, 0.2199, 0.2201, 0.4999, 0.5001, 1.2999, 1.3001, 2.3499, 2.3501])
+def test_plain_form_at_its_series_lengths(x):
+    """Candidates outside the fixed-point ranges (a drift above f0/1024, or f above 1.3 f*) on both sides of
+    each length of the link-transfer series."""
+    T, N, n = wk.YEAR, 64, 9
+    eta = 2.0 / 1024 if x < 1.3 else 0.0
+    f0 = x * FSTAR / (1.0 + eta)           # x = f_max / f*
+    th = candidates(f0, eta * f0 / T, n, int(1e4 * x))
+    out = api.Context(T).waveform_aet(torch.as_tensor(th, device="cuda"), N)
+    q, ref = ld.template_aet(th, N, T)
+    assert np.array_equal(out[3].cpu().numpy(), q)
+    norm = lambda y: np.sqrt((np.abs(y) ** 2).sum(1).astype(np.float64))  # noqa: E731
+    for h, r in zip(out[:2], ref[:2]):
+        assert np.all(norm(h.cpu().numpy() - r) <= tolerance(th, T) * norm(r))
