@@ -44,6 +44,15 @@ int tile_size(gb_ctx* ctx, int64_t total, int warps) {
     return (int)t;
 }
 
+// FP64 likelihood: CTAs of four warps, at most 16 candidates per warp, what a
+// warp sets up at a time (160,000 candidates: 3.91 ms; 8 or 32 per warp: 4.03
+// ms).  Every entry point that uses the FP64 plan of a layout asks for this
+// one, so that they share it.
+int tile_size64(gb_ctx* ctx, int64_t total) {
+    if (ctx->tune_tile64 > 0) return std::min(ctx->tune_tile64, 128);
+    return std::min(tile_size(ctx, total, 4), 64);
+}
+
 int loglik_impl(gb_ctx_t* ctx, const char* name, int prec, const gb_window_t* win, int32_t n_win, const double* dA,
                 const double* dE, const double* wA, const double* wE, int64_t n_bins, const double* theta,
                 int64_t n_rows, double* logL, double* dh, double* dh_im, double* hh, void* stream,
@@ -58,18 +67,13 @@ int loglik_impl(gb_ctx_t* ctx, const char* name, int prec, const gb_window_t* wi
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_error(ctx, e, "loglik: cudaSetDevice");
     const Plan* plan = nullptr;
-    const int warps = 4;
     // mixed: work items of at most 16 candidates (one warp each; smaller
     // items balance the persistent warps' tails), fewer when the batch would
     // not give every resident warp of the GPU one item
     int item = (int)std::min<int64_t>(16, std::max<int64_t>(1, (total + sm_count(ctx) * 16 - 1) / (sm_count(ctx) * 16)));
     if (ctx->tune_item > 0) item = std::min(ctx->tune_item, 32);
     if (dT) item = std::min(item, 16);   // the T-channel kernel's items hold at most 16 candidates
-    // FP64: tiles of at most 16 candidates per warp, what a warp sets up at a
-    // time (160,000 candidates: 3.91 ms; 8 or 32 per warp: 4.03 ms)
-    int tile = std::min(tile_size(ctx, total, warps), 16 * warps);
-    if (ctx->tune_tile64 > 0) tile = std::min(ctx->tune_tile64, 32 * warps);
-    rc = get_plan(ctx, prec, win, n_win, prec == GB_MIXED ? item : tile, &plan);
+    rc = get_plan(ctx, prec, win, n_win, prec == GB_MIXED ? item : tile_size64(ctx, total), &plan);
     if (rc != GB_OK) return rc;
     if (prec == GB_FP64)
         return launch_loglik_fp64(ctx, *plan, dA, dE, wA, wE, theta, logL, dh, hh, dh_im, dT, wT,
@@ -268,7 +272,7 @@ int gb_loglik_rows(gb_ctx_t* ctx, const gb_window_t* win, int32_t n_win, const d
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_error(ctx, e, "gb_loglik_rows: cudaSetDevice");
     const Plan* plan = nullptr;
-    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size(ctx, total, 4), &plan);
+    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size64(ctx, total), &plan);
     if (rc != GB_OK) return rc;
     int nc_max = 0;
     for (int i = 0; i < n_win; ++i) nc_max = std::max(nc_max, win[i].n_cand);
@@ -355,7 +359,7 @@ int gb_mh_certified(gb_ctx_t* ctx, const gb_window_t* win, int32_t n_win, const 
     cs.n_flip = cs.n_new + passes;
     // the FP64 plan of this layout holds the device copy of the windows
     const Plan* plan64 = nullptr;
-    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size(ctx, total, 4), &plan64);
+    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size64(ctx, total), &plan64);
     if (rc != GB_OK) return rc;
     const gb_window_t* d_win = plan64->d_win;
     const int n_max = plan64->n_max;
@@ -415,7 +419,7 @@ int gb_snr_multi(gb_ctx_t* ctx, const gb_window_t* win, int32_t n_win, const dou
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_error(ctx, e, "gb_snr_multi: cudaSetDevice");
     const Plan* plan = nullptr;
-    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size(ctx, std::max<int64_t>(total, 1), 4), &plan);
+    rc = get_plan(ctx, GB_FP64, win, n_win, tile_size64(ctx, total), &plan);
     if (rc != GB_OK) return rc;
     return launch_multi_gram(ctx, plan->d_win, n_win, plan->n_max, (dh || rho) ? dA : nullptr, dE, wA, wE, theta,
                              kmax, gram, dh, rho, (cudaStream_t)stream);

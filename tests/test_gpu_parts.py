@@ -148,3 +148,36 @@ def test_time_budget_leaves_the_preparation_out(grad):
     for a, b in zip(long(), ref):
         assert torch.equal(a, b)
     ctx.check()
+
+
+def test_entry_points_share_a_layouts_fp64_plan():
+    """A plan cannot be made while a stream is captured; the likelihood's serves
+    the listed rows, the certified round and the Gram matrices of its layout."""
+    n = 24000
+    wins, d, w, th = _args("loglik", n, 4)
+    win, th = wins[1][:4] + (0, n), th[n:2 * n].clone()
+    ctx = api.Context(wk.YEAR)
+    rows = torch.arange(n, dtype=torch.int32, device="cuda")
+    lo, hi = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.full((1,), 100, dtype=torch.int32, device="cuda")
+    zero = torch.zeros((1, n), dtype=torch.float64, device="cuda")
+    log_u = torch.log(torch.rand((1, n), dtype=torch.float64, device="cuda"))
+    one = torch.ones(1, dtype=torch.float64, device="cuda")
+    pairs = [wins[1][:4] + (2 * k, 2) for k in range(n // 2)]
+    other = [(win[0] + 1,) + win[1:]]
+    ctx.mh_certified(other, *d, *w, th, zero, log_u, one)   # scratch of this size
+    for lay in ([win], pairs):
+        for prec in ("fp64", "mixed"):
+            ctx.loglik(lay, *d, *w, th, prec=prec)
+    want = ctx.loglik([win], *d, *w, th)[0][:100].clone()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            got = ctx.loglik_rows([win], *d, *w, th, rows, lo, hi)[0]
+            pending = ctx.mh_certified([win], *d, *w, th, zero, log_u, one)[-1]
+            rho = ctx.snr_multi(pairs, *d, *w, th)[0]
+        graph.replay()
+    stream.synchronize()
+    assert torch.equal(got[:100], want) and int(pending) == 0
+    assert torch.equal(rho, ctx.snr_multi(pairs, *d, *w, th)[0])
