@@ -252,8 +252,8 @@ def flops_per_grad_fp64(N, f_hz, T):
 def flops_per_eval_fp64(N, f_hz, T):
     """Floating-point operations of one evaluation of the FP64 path (FMA = 2,
     a sincos or sincospi counted as 20), counted from the algorithm as its
-    double form states it (the fixed-point form computes the same quantities).  Per sample: three receiver phases (projection 6,
-    phase in cycles 18, reduction and sincospi 22) 138; f and a 4; three arms
+    double form states it (the fixed-point form computes the same quantities).
+    Per sample: three receiver phases (projection 6, phase in cycles 18, reduction and sincospi 22) 138; f and a 4; three arms
     (k.n 5, n.H.n 19, two links of 20 + 4 J each: argument, series in
     -4X^2, complex scaling and two complex products) 3 x (64 + 8 J); the delay
     factor by its short series and D^2, 27; X, Y, Z with (1 - D^2) 72; the A/E
@@ -270,6 +270,38 @@ def fp64_peak_tflops(clock_mhz=2070.0):
     Two lanes per SM (1/64 of the 128 FP32 lanes) is what GB300's nominal
     1.25 TFLOP/s dense FP64 implies at 2.07 GHz."""
     return 152 * 2 * 2 * clock_mhz * 1e6 / 1e12
+
+
+def products_fp64(N, f_hz, grad=False):
+    """32 x 32 -> 64-bit integer products of one evaluation (or gradient) of the
+    FP64 path in its fixed-point form, A and E, counted by running the headers
+    on the host: a sample takes 485 (541 above f*/2) and its reverse sweep 967
+    (1,047); a transform 12 per complex product, 9 N per two stages after the
+    first two and 6 N for an odd last one, of both channels, twice for a
+    gradient.  Other integer and all FP64 work is left out."""
+    high = f_hz / (299792458.0 / (2 * math.pi * 2.5e9)) > 0.5
+    stages = int(math.log2(N)) - 2
+    fft = 2 * N * (9 * (stages // 2) + 6 * (stages % 2))
+    if not grad:
+        return N * (541 if high else 485) + fft
+    return N * ((541 + 1047) if high else (485 + 967)) + 2 * fft
+
+
+def product_peak(clock_mhz=2070.0):
+    """32 x 32 -> 64-bit products a second, in 1e12: 152 SMs x 4 schedulers x
+    one warp instruction of 32 per 4 clocks (measured)."""
+    return 152 * 4 * 8 * clock_mhz * 1e6 / 1e12
+
+
+def fp64_roofline(products, tflop, ms, kernel, profile):
+    """The fixed-point FP64 kernels against the unit that does their work; beside
+    it the same work as double operations and the FP64 pipe's peak."""
+    rate = products / (ms / 1e3) / 1e12
+    return {"bound": "alu", "achieved": rate, "peak": product_peak(), "unit": "T products/s",
+            "frac": rate / product_peak(), "traffic": profiled_traffic(profile), "kernel": kernel,
+            "as_double_tflops": tflop / (ms / 1e3) / 1e12, "fp64_peak_tflops": fp64_peak_tflops(),
+            "peak_note": "32 x 32 -> 64-bit integer products from unit counts: 152 SM x 4 schedulers x 32 lanes per "
+                         "4 clocks x 2070 MHz; achieved counts the products of the 64-bit fixed-point form only"}
 
 
 def cpu_model():
@@ -512,17 +544,11 @@ def run_workload(args):
             "peak_note": "FP32 FMA peak from unit counts: 152 SM x 128 lanes x 2 x 2070 MHz; the timed call "
                          "is the preparation kernel and the gradient kernel"}
         gflops64 = sum(512 * flops_per_grad_fp64(w[2], f, wl.T) for w, f in zip(wl.windows, f_mid))
+        prod64 = sum(512 * products_fp64(w[2], f, grad=True) for w, f in zip(wl.windows, f_mid))
         line["grad_fp64"] = {"value": 512 * len(sub) / ms_g64 * 1e3, "unit": "gradients/s", "ms": ms_g64,
                              "sample": "512 candidates per window",
-                             "roofline": {"bound": "alu", "achieved": gflops64 / (ms_g64 / 1e3) / 1e12,
-                                          "peak": fp64_peak_tflops(), "unit": "TFLOP/s",
-                                          "frac": gflops64 / (ms_g64 / 1e3) / 1e12 / fp64_peak_tflops(),
-                                          "traffic": profiled_traffic("grad_fp64_population"),
-                                          "kernel": "grad64_kernel",
-                                          "peak_note": "FP64 peak from unit counts: 152 SM x 2 FP64 FMA lanes x 2 "
-                                                       "x 2070 MHz; achieved counts the reverse-mode work as "
-                                                       "double operations, which the kernel does in 64-bit fixed "
-                                                       "point on the integer pipe, so the fraction passes 1"}}
+                             "roofline": fp64_roofline(prod64, gflops64, ms_g64, "grad64_kernel",
+                                                       "grad_fp64_population")}
         boxes = np.array([np.concatenate([wl.theta[c:c + m].min(0), wl.theta[c:c + m].max(0)])
                           for (_, _, _, _, c, m) in wl.windows])
         ga_ms = {}
@@ -908,7 +934,7 @@ def main():
     flops64 = sum(n * flops_per_eval_fp64(w[2], f, wl.T) for w, f in zip(wl.windows, f_mid))
     fp32_peak = 152 * 128 * 2 * 2070e6 / 1e12
     achieved = flops / (kern_only_mx / 1e3) / 1e12
-    achieved64 = flops64 / (kern_64 / 1e3) / 1e12
+    prod64 = sum(n * products_fp64(w[2], f) for w, f in zip(wl.windows, f_mid))
     # Alg. 4 with its temperature ladder (15, 10, 5, 3, 2, 1): six rounds of
     # 10,000 device-drawn proposals per window, Gaussian refits between rounds
     from paper_2307_03763_gb300.posterior import AnnealedPosterior
@@ -987,14 +1013,7 @@ def main():
         "annealed_posterior_6T_kde": annealed_kde,
         "fp64": {"value": value64, "unit": UNIT, "steps": fp64_steps, "ms_per_step": tot_64 / fp64_steps,
                  "s_per_10k_posterior": tot_64 / fp64_steps / 1e3 / nwin, "loglik_ms": kern_64,
-                 "roofline": {"bound": "alu", "achieved": achieved64, "peak": fp64_peak_tflops(),
-                              "unit": "TFLOP/s", "frac": achieved64 / fp64_peak_tflops(),
-                              "traffic": profiled_traffic("loglik_fp64_posterior"),
-                              "kernel": "loglik64_kernel",
-                              "peak_note": "FP64 peak from unit counts: 152 SM x 2 FP64 FMA lanes x 2 x 2070 MHz "
-                                           "(the nominal 1.25 TFLOP/s dense FP64); achieved counts double operations, which "
-                                           "the kernel does in 64-bit fixed point on the integer pipe, so the fraction "
-                                           "passes 1"}},
+                 "roofline": fp64_roofline(prod64, flops64, kern_64, "loglik64_kernel", "loglik_fp64_posterior")},
         "mixed_vs_fp64": {"max_abs_dlogL": float(dl.max()), "p99_abs_dlogL": float(dl.quantile(0.99)),
                           "median_abs_dlogL": float(dl.median()), "snr_range": [20, 200],
                           "by_proposal_snr": by_snr},

@@ -58,8 +58,14 @@ extern "C" {
 #define GB_ENOMEM   -4   /* device allocation failed */
 
 #define GB_FP64   0      /* double precision: set-up, inner products and outputs in IEEE
-                            double; response samples and FFT in 64-bit fixed point (58 or
-                            more fractional bits) where the parameters allow, else double */
+                            double.  Where the parameters allow, the response samples and
+                            the transforms are in 64-bit fixed point: phases and response
+                            factors with 57 or more fractional bits, their sums and the
+                            samples with 52 (49 at N = 1,024) of the channels' scale, a
+                            gradient's residual and its transform to 2^-60 of the sum of the
+                            residual's moduli; the chirp's differences between the receivers
+                            (below 1e-8 rad) to 2^-29 of themselves, and their derivatives in
+                            float.  Else every step in double */
 #define GB_MIXED  1      /* carrier phase modulo one cycle in 64-bit fixed point
                             (double-word float arithmetic for candidates outside
                             its ranges), per-candidate set-up and carrier offset
@@ -129,6 +135,9 @@ int gb_ctx_set_time_budget(gb_ctx_t* ctx, double seconds);
  * gb_loglik_phase, gb_loglik_phase_aet with GB_MIXED, or gb_mh_certified)
  * records `start` on its stream after the window preparation, just before
  * those kernels, and `end` just after them; the context then forgets both.
+ * `start` between them keeps the first of the kernels from starting beside
+ * the preparation, as it does otherwise: the interval is the kernels' alone,
+ * the call as a whole some microseconds longer.
  * NULL for both clears them.  GB_EINVAL if exactly one is NULL. */
 int gb_ctx_set_kernel_events(gb_ctx_t* ctx, void* start, void* end);
 

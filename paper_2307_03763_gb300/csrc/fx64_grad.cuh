@@ -352,7 +352,7 @@ struct FinGFx {
     double F;      // scale of everything but A's row, less the normalisation of the cotangents
     double FA;     // scale of A's row
 };
-GB_FX void setup_fin(const double* th, double T, double arm_c, int lg, const FxTrig& t, double si, FinGFx& c) {
+GB_FX void setup_fin(const double* th, double arm_c, int lg, const FxTrig& t, double si, FinGFx& c) {
     const double pi = 3.14159265358979323846;
     c.f0 = th[0];
     c.a0 = pi * th[0] * arm_c;
@@ -375,7 +375,6 @@ GB_FX void setup_fin(const double* th, double T, double arm_c, int lg, const FxT
     c.gxp[1] = 4.0 * Ax * t.s2;
     c.FA = 2.0 / (double)(1 << lg) * (8.0 * c.a0 * t.sa * t.ca) * 0.70710678118654752;
     c.F = c.FA * th[4];
-    (void)T;
 }
 // gradient from the sums; norm: the cotangents' value per unit (2^-60 of an integer)
 GB_FX void finish_gfx(const FinGFx& c, double T, const double* s, double norm, double* grad) {

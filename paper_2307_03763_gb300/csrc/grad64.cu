@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(kWarpsG * 32, kMinCtasG) grad64_kernel(
             setup_lane(th, g, c.t, t, si);
             if (c.t.tier >= 0 && !setup_gfx(th, T, g.arm_c, t, c.g)) c.t.tier = -1;
             if (c.t.tier >= 0) {
-                setup_fin(th, T, g.arm_c, g.logN, t, si, c.fin);
+                setup_fin(th, g.arm_c, g.logN, t, si, c.fin);
             } else if (!c.t.bad) {
                 setup_grad(th, T, g.inv_fstar, __dadd_rn(__dmul_rn(th[0], T), -(double)c.t.q), c.d);
             }

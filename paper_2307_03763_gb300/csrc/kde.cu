@@ -105,7 +105,7 @@ __device__ __forceinline__ double sum_ranks(const double* v) {
 // over the eight): CTA r holds partial sums 32 r .. 32 r + 31, so the FP64 work
 // and the gathers spread over eight SMs.  Counts go to the CTA that owns the
 // cell's row block by distributed-shared-memory atomics.  16 windows of 10,000
-// entries, grid 64: 79 us (332 us for one CTA per pair: a division per entry,
+// entries, grid 64: 80 us (332 us for one CTA per pair: a division per entry,
 // serial exponentials, one SM's FP64 pipe).
 __global__ void __cluster_dims__(kKdeCtas, 1, 1) __launch_bounds__(kKdeThreads)
     kde_build_kernel(int n, int G, const double* __restrict__ theta, const int32_t* __restrict__ chain,

@@ -108,7 +108,7 @@ void host_gradients(int B, const double* theta, const double* delta, double T, d
         setup_fx(th, T, arm_c, delta[b], lg, t, c);
         tier[b] = c.tier;
         if (c.tier < 0 || !setup_gfx(th, T, arm_c, t, cg)) continue;
-        setup_fin(th, T, arm_c, lg, t, sin(th[5]), fin);
+        setup_fin(th, arm_c, lg, t, sin(th[5]), fin);
         double sums[kGSums];
         const fx* g = cot + (size_t)b * 6 * (1 << lg);
         if (c.tier == 0) sweep<0>(c, cg, tw, geo, arm_c, lg, g, sums);
