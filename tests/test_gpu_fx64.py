@@ -169,3 +169,43 @@ def test_plain_form_at_its_series_lengths(x):
     norm = lambda y: np.sqrt((np.abs(y) ** 2).sum(1).astype(np.float64))  # noqa: E731
     for h, r in zip(out[:2], ref[:2]):
         assert np.all(norm(h.cpu().numpy() - r) <= tolerance(th, T) * norm(r))
+
+
+@pytest.mark.parametrize("f0,fdot", [(15e-3, 1.2e-13), (23e-3, 2e-13)])
+def test_gradients_beside_a_loud_bin(f0, fdot):
+    """N = 1,024 against differences of fourth order of the long-double model,
+    steps of 1e-4 rad of phase.  Samples carry 2^-49 of the channels' scale (8
+    units of 2^-52), the response, the transforms and the sums a few units
+    each: 32 units of 2^-52 of the gradient's norm in all."""
+    T, N, n = wk.YEAR, 1024, 3
+    th = candidates(f0, fdot, n, int(1e4 * f0))
+    th[:, 2] = [0.3, -0.8, 1.1]
+    q, h = ld.template_aet(th, N, T)
+    rng = np.random.default_rng(N)
+    win = (int(q[0]) - N // 2, N, N)
+    d = [(rng.standard_normal(N) + 1j * rng.standard_normal(N)) * 1e-20 for _ in range(2)]
+    for x in d:
+        x[N // 2 + 3] = 1e3 * np.abs(x).max()
+    w = [rng.uniform(0.5, 1.5, N) * 1e41 for _ in range(2)]
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), device="cuda")  # noqa: E731
+    _, g = api.Context(T).loglik_grad([win + (0, 0, n)], dev(d[0]), dev(d[1]), dev(w[0]), dev(w[1]), dev(th))
+    j = q[:, None] - N // 2 + np.arange(N)[None, :] - win[0]
+    ok, jc = (j >= 0) & (j < N), np.clip(j, 0, N - 1)
+
+    def value(step):
+        total = 0
+        for x, wt, s in zip(d, w, ld.template_aet(th, N, T, step)[1]):
+            x, wt = x.astype(np.clongdouble)[jc], wt.astype(np.longdouble)[jc] * ok
+            total = total + (wt * ((x * s.conj()).real - (s.real ** 2 + s.imag ** 2) / 2)).sum(1)
+        return total * (4 / np.longdouble(T))
+
+    unit = 1 / np.concatenate([[2 * math.pi * T, math.pi * T * T], [2 * math.pi * f0 * 500] * 2, [1.0, 2.0, 4.0, 1.0]])
+    unit = np.tile(unit.astype(np.longdouble), (n, 1))
+    unit[:, 4] = th[:, 4]
+    ref = np.empty((n, 8), np.longdouble)
+    for k in range(8):
+        e = np.zeros(8, np.longdouble)
+        e[k] = 1e-4 * unit[:, k].min()
+        ref[:, k] = (8 * (value(e) - value(-e)) - (value(2 * e) - value(-2 * e))) / (12 * e[k])
+    err = np.abs((g.cpu().numpy() - ref) * unit).max(1) / np.sqrt(((ref * unit) ** 2).sum(1))
+    assert err.max() < 32 * 2.0 ** -52, err
